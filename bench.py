@@ -186,8 +186,11 @@ def kernel_source_hash():
     removed: it changes when the code changes, not when a comment does."""
     import re
     h = hashlib.sha256()
-    for f in ("k_block.cuh", "k_block_inst.cuh", "iter_math.cuh", "ofv_common.cuh"):
-        with open(os.path.join(ROOT, "paper_2509_25924_gb300", "csrc", f)) as fh:
+    for f in ("k_walk.cuh", "k_block.cuh", "k_block_inst.cuh", "iter_math.cuh", "ofv_common.cuh"):
+        path = os.path.join(ROOT, "paper_2509_25924_gb300", "csrc", f)
+        if not os.path.exists(path):
+            continue
+        with open(path) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         lines = (re.sub(r"//.*$", "", ln).rstrip() for ln in src.splitlines())
         h.update("\n".join(ln for ln in lines if ln).encode())

@@ -114,8 +114,9 @@ typedef struct {
                            (48 for KR <= 5, 64 for KR 6..10); or the alternative, 32.  With 0,
                            ofv_compute_batched's autotuner picks one of
                            the two per batch signature (ofv_batch_tuning reports it); nonzero fixes it.
-                           The window sums' rounding follows the tile grid, so fields of different tile
-                           edges agree to FP32 rounding, not bitwise.  The estimator variants (Gaussian
+                           The edge is the unit of rows of a strip and selects the larger or the smaller
+                           tiles; the order of a pixel's window sums follows its position in the image,
+                           so all tiles give the same field bitwise.  The estimator variants (Gaussian
                            window, increment form, region mask) and the reverse mode run the default. */
 } ofv_params;
 
@@ -340,14 +341,13 @@ typedef struct {
  * Sec. 2 (steps 1-6, Eq. 2) for every pair, as ofv_compute computes it.
  * pairs is a HOST array.  All 2n frames are ingested by one launch and each
  * pyramid level of all of them is reduced by one launch; then every (level,
- * iteration, tile) of every pair runs in ONE persistent launch of the fused
- * kernel: CTAs take work units from a queue in the order of a schedule, and
+ * iteration, tile) of every pair runs in ONE launch of the fused kernel: one
+ * CTA per work unit, which it takes from a queue in the order of a schedule;
  * a unit of one Gauss-Newton iteration waits (bounded) until the previous
  * iteration of its pair is complete.  The first batch of a given signature
  * (sorted sizes and parameters) runs the autotuner: each candidate -- tile
  * shape (see ofv_params.tile_edge), schedule (all pairs stage by stage, or
- * groups of 8 pairs) and persistent grid (the resident CTAs per SM, or one
- * fewer) -- is timed on the batch itself and the fastest is kept
+ * groups of 8 pairs) -- is timed on the batch itself and the fastest is kept
  * for later batches of that signature (that first call waits for its
  * timings).  Otherwise the call enqueues the batch on s and returns; the
  * fields are valid once s reaches them, and the next call's host work
@@ -362,18 +362,18 @@ typedef struct {
 ofv_status ofv_compute_batched(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_t s);
 
 /* Configuration used by the last ofv_compute_batched call: schedule (0 =
- * stage-major over all pairs, else group size), persistent CTAs per SM, the
+ * stage-major over all pairs, else group size), resident CTAs per SM, the
  * output tile edge of the block kernel in px (with ofv_params.tile_edge = 0
  * the autotuner tries the radius's default and alternative edges, except
  * with the Gaussian window or the increment form, which have the default
  * only; a nonzero tile_edge fixes the edge),
- * duration of its persistent launch in ms, and whether that call tuned.  A
+ * duration of its launch in ms, and whether that call tuned.  A
  * handle created with tile_edge set to the reported edge computes, through
  * ofv_compute, bitwise the fields the batch computed. */
 ofv_status ofv_batch_tuning(const ofv_handle *h, int *schedule, int *ctas_per_sm, int *tile_edge, double *ms,
                             int *tuned);
 
-/* Test hook for the bounded waits of the persistent launch: runs one CTA
+/* Test hook for the bounded waits of the batched launch: runs one CTA
  * whose work unit depends on a counter nothing increments.  Expected result:
  * OFV_ERR_TIMEOUT after about timeout_us, *error_word = 1 (the device word),
  * the same value in the mapped host word that asynchronous batches report
@@ -425,7 +425,7 @@ ofv_status ofv_graph_destroy(ofv_graph *g);
 /* The batched form for camera streams of uneven size (Sec. 6: several
  * cameras or streams at fixed rates): records ofv_compute_batched(h, n,
  * pairs) -- the ingest and reduce launches of every frame and the one
- * persistent launch of all (level, iteration, tile) units -- into a CUDA
+ * launch of all (level, iteration, tile) units -- into a CUDA
  * graph, so a new set of pairs written into the same buffers costs one
  * ofv_graph_launch and no host work.  pairs is a HOST array as for
  * ofv_compute_batched; its buffers are the ones every launch reads and

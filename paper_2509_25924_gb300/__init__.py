@@ -295,7 +295,7 @@ def _pair_array(pairs):
 
 def ofv_compute_batched(h: int, pairs, stream=None):
     """pairs: sequence of (I1, I2, u, v) CUDA tensors (each H x W) or Pair
-    structures; all pairs of the batch run in one persistent launch."""
+    structures; all pairs of the batch run in one launch."""
     arr = _pair_array(pairs)
     _check(_lib.ofv_compute_batched(h, len(pairs), ctypes.cast(arr, ctypes.c_void_p), _stream(stream)),
            "ofv_compute_batched")

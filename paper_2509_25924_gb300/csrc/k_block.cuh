@@ -1,7 +1,9 @@
-// Block-tiled fused Gauss-Newton iteration (Sec. 2 step 3, Eq. 2), the
-// kernel behind OFV_PATH_FUSED for window radii 1..10.
+// Fused Gauss-Newton iteration (Sec. 2 step 3, Eq. 2) for window radii
+// 1..10: launch descriptors, shared-memory and TMA primitives, and the tile
+// body of the estimator variants (Gaussian window, increment form, region
+// mask).  The box window's body is in k_walk.cuh.
 //
-// One CTA owns a TS x TS tile of output pixels (by default 48 px for
+// The variants' CTA owns a TS x TS tile of output pixels (by default 48 px for
 // KR <= 5 and 64 for KR 6..10; see block_tile_edge) and works
 // entirely on chip in five phases:
 //   0. stage the two level images over the tile, its KR window halo, a
@@ -42,23 +44,23 @@ struct BlockParams {
     int mode;                    // V0Mode, uniform per launch
     int use_tma;                 // 1: tm[k] maps the two level images of pair k
     int *err;                    // error word (set to 1 when a TMA wait expires), or null
-    int by0;                     // first tile row of the launch (blockIdx.y + by0)
+    int row0, row1;              // output rows of the launch (row0 a multiple of the radius's tile edge)
     CUtensorMap tm[kBlockMaxBatch][2];
 };
 
 // The block kernels' templates take KS = KR + 16 V + 32 Q: the window radius
 // KR (1 .. 10), the tile shape V (0: the default shape of the radius, 1: its
 // alternative, which the batched autotuner tries and ofv_params.tile_edge
-// selects) and Q = 1 for the persistent batched kernel, which runs 48-px
-// tiles with 512 threads instead of 576 (its queue state leaves fewer
-// registers: 576 threads spill there, +3.2 % with 512).  Each output pixel
+// selects) and Q = 1 for the variants' batched kernel, which runs 48-px
+// tiles with 512 threads instead of 576.  Each output pixel
 // is computed by the same tile with the same arithmetic whatever the thread
 // count, so the two kernels give the same fields.
 __host__ __device__ constexpr int ks_radius(int ks) { return ks & 15; }
 __host__ __device__ constexpr int ks_shape(int ks) { return (ks >> 4) & 1; }
 __host__ __device__ constexpr int ks_queue(int ks) { return ks >> 5; }
 
-// Output tile edge of shape v for radius kr.  Default shapes, measured per
+// Output tile edge of shape v for radius kr: of the variants' tiles, and the
+// unit of rows of a strip.  Default shapes, measured per
 // radius (1 Mp stream, fields/s): KR <= 5: 48-px tiles of 576 threads, two
 // CTAs per SM, 56 registers (512 threads: -2 %; 640: no gain, 48 registers
 // and spills; 64-px tiles at one CTA per SM: -15..-18 %); KR 6..10: 64-px
@@ -68,6 +70,17 @@ __host__ __device__ constexpr int ks_queue(int ks) { return ks >> 5; }
 __host__ __device__ constexpr int block_tile_edge(int kr, int v)
 {
     return v == 0 ? (kr <= 5 ? 48 : 64) : 32;
+}
+
+// Output tile of the box-window kernels (k_walk.cuh), which give the same
+// field whatever their tiles: the default and the smaller alternative.
+__host__ __device__ constexpr int walk_tile_w(int kr, int v)
+{
+    return kr <= 4 ? 56 : v == 0 ? (kr == 5 ? 48 : 64) : kr <= 8 ? 48 : 40;
+}
+__host__ __device__ constexpr int walk_tile_h(int kr, int v)
+{
+    return kr <= 4 ? (v == 0 && kr > 2 ? 40 : 24) : v == 0 ? (kr == 5 ? 48 : 64) : 32;
 }
 
 template <int KS> struct BlockShape {
@@ -160,9 +173,13 @@ __device__ __forceinline__ long long global_ns()
 // mbarrier and TMA (bulk tensor copy) primitives, CTA scope.
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
+// N barriers of count 1, fenced together.
+template <int N>
+__device__ __forceinline__ void mbar_init_n(uint64_t *bar)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+#pragma unroll
+    for (int b = 0; b < N; ++b)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + b)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -302,33 +319,6 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b)
 struct Sample2 { float2 val, gx, gy; };
 
 // Bilinear value and doubled gradient (undivided central differences) of a
-// staged 4x4 neighbourhood, for the two frames at once: rm1, rm2 point at
-// the tap left of column x0 in row y0-1 of each frame's staged tile; f_x,
-// f_y hold each frame's fractions.  Interpolation as a + f (b - a); the
-// row interpolation of the column differences equals the difference of row
-// interpolations (gy).  Each lane rounds as the scalar operations would.
-template <typename T, int SP>
-__device__ __forceinline__ Sample2 bilin_staged2(const T *__restrict__ rm1, const T *__restrict__ rm2, float2 f_x,
-                                                 float2 f_y)
-{
-    auto ld2 = [&](int off) { return make_float2(to_f(rm1[off]), to_f(rm2[off])); };
-    const float2 e0 = ld2(1), e1 = ld2(2);
-    const float2 q00 = ld2(SP), q01 = ld2(SP + 1), q02 = ld2(SP + 2), q03 = ld2(SP + 3);
-    const float2 q10 = ld2(2 * SP), q11 = ld2(2 * SP + 1), q12 = ld2(2 * SP + 2), q13 = ld2(2 * SP + 3);
-    const float2 e2 = ld2(3 * SP + 1), e3 = ld2(3 * SP + 2);
-    Sample2 s;
-    const float2 v0 = fma2(f_x, sub2(q02, q01), q01), v1 = fma2(f_x, sub2(q12, q11), q11);
-    s.val = fma2(f_y, sub2(v1, v0), v0);
-    const float2 da0 = sub2(q02, q00), db0 = sub2(q03, q01), da1 = sub2(q12, q10), db1 = sub2(q13, q11);
-    const float2 gx0 = fma2(f_x, sub2(db0, da0), da0), gx1 = fma2(f_x, sub2(db1, da1), da1);
-    s.gx = fma2(f_y, sub2(gx1, gx0), gx0);
-    const float2 vm = fma2(f_x, sub2(e1, e0), e0), vp = fma2(f_x, sub2(e3, e2), e2);
-    const float2 gy0 = sub2(v1, vm), gy1 = sub2(vp, v0);
-    s.gy = fma2(f_y, sub2(gy1, gy0), gy0);
-    return s;
-}
-
-// Bilinear value and doubled gradient (undivided central differences) of a
 // staged 4x4 neighbourhood for the two frames at once, with each
 // interpolation written (1 - f) a + f b, which is exact at f = 0 and f = 1:
 // a sample taken at the tap to the left with fraction 1 equals the sample at
@@ -361,7 +351,7 @@ __device__ __forceinline__ Sample2 bilin_weighted2(const T *__restrict__ rm1, co
 // integer offset (ix, iy) with fractions (fx2, fy2), frame 1 at -(ix, iy) - 1
 // with fractions 1 - (fx2, fy2); base indexes the staged element left of and
 // above the pixel.
-template <typename T, int SP, bool VAR>
+template <typename T, int SP>
 __device__ __forceinline__ void products_staged(const T *__restrict__ st1, const T *__restrict__ st2, int base, int ix,
                                                 int iy, float fx2, float fy2, const IterArgs &a, float2 V0, float p[5])
 {
@@ -373,7 +363,7 @@ __device__ __forceinline__ void products_staged(const T *__restrict__ st1, const
     const float Gx = 0.25f * (s12.gx.x + s12.gx.y);
     const float Gy = 0.25f * (s12.gy.x + s12.gy.y);
     const float It = s12.val.y - s12.val.x;
-    const float r = (VAR && a.inc) ? -It : Gx * V0.x + Gy * V0.y - It;
+    const float r = a.inc ? -It : Gx * V0.x + Gy * V0.y - It;
     p[0] = Gx * Gx;
     p[1] = Gx * Gy;
     p[2] = Gy * Gy;
@@ -389,7 +379,7 @@ __device__ __forceinline__ void products_staged(const T *__restrict__ st1, const
 // unless a component of h is an integer, where the weight 1 on the next tap
 // gives the same sample exactly.  Both stencils then lie within REACH + 1 px
 // and one integer test checks both.  Farther warps take the general sampler.
-template <typename T, int SP, bool VAR = false>
+template <typename T, int SP>
 __device__ __forceinline__ void products_interior(const T *__restrict__ st1, const T *__restrict__ st2, int sx0,
                                                   int sy0, const IterArgs &a, int x, int y, float2 V0, float p[5])
 {
@@ -397,7 +387,7 @@ __device__ __forceinline__ void products_interior(const T *__restrict__ st1, con
     const float flx = floorf(hx), fly = floorf(hy);
     const int ix = (int)flx, iy = (int)fly;
     if (((unsigned)(ix + kBlockReach) | (unsigned)(iy + kBlockReach)) < (unsigned)(2 * kBlockReach)) {
-        products_staged<T, SP, VAR>(st1, st2, (y - 1 - sy0) * SP + (x - 1 - sx0), ix, iy, hx - flx, hy - fly, a, V0,
+        products_staged<T, SP>(st1, st2, (y - 1 - sy0) * SP + (x - 1 - sx0), ix, iy, hx - flx, hy - fly, a, V0,
                                     p);
     } else {
         const T *P1 = static_cast<const T *>(a.P1), *P2 = static_cast<const T *>(a.P2);
@@ -405,7 +395,7 @@ __device__ __forceinline__ void products_interior(const T *__restrict__ st1, con
         const Sample s2 = sample_global(P2, a.H, a.W, a.pitch, x, y, hx, hy);
         const float Gx = 0.5f * (s1.gx + s2.gx), Gy = 0.5f * (s1.gy + s2.gy);
         const float It = s2.val - s1.val;
-        const float r = (VAR && a.inc) ? -It : Gx * V0.x + Gy * V0.y - It;
+        const float r = a.inc ? -It : Gx * V0.x + Gy * V0.y - It;
         p[0] = Gx * Gx;
         p[1] = Gx * Gy;
         p[2] = Gy * Gy;
@@ -418,7 +408,7 @@ __device__ __forceinline__ void products_interior(const T *__restrict__ st1, con
 // products of an in-reach stand-in offset, when the warp leaves the staged
 // margin; the caller then recomputes the pixel with products_interior.
 // Keeps the hot loop free of a divergent branch and a call.
-template <typename T, int SP, bool VAR = false>
+template <typename T, int SP>
 __device__ __forceinline__ bool products_staged_only(const T *__restrict__ st1, const T *__restrict__ st2, int sx0,
                                                      int sy0, const IterArgs &a, int x, int y, float2 V0, float p[5])
 {
@@ -426,7 +416,7 @@ __device__ __forceinline__ bool products_staged_only(const T *__restrict__ st1, 
     const float flx = floorf(hx), fly = floorf(hy);
     const int ix = (int)flx, iy = (int)fly;
     const bool near = ((unsigned)(ix + kBlockReach) | (unsigned)(iy + kBlockReach)) < (unsigned)(2 * kBlockReach);
-    products_staged<T, SP, VAR>(st1, st2, (y - 1 - sy0) * SP + (x - 1 - sx0), near ? ix : 0, near ? iy : 0, hx - flx,
+    products_staged<T, SP>(st1, st2, (y - 1 - sy0) * SP + (x - 1 - sx0), near ? ix : 0, near ? iy : 0, hx - flx,
                                 hy - fly, a, V0, p);
     return near;
 }
@@ -463,10 +453,10 @@ __host__ __device__ constexpr int first_iter_of_band_up(int b)
 // With bars (TMA staging in three bands), the loop waits for band b just
 // before the first iteration that can touch it, so the first rows of
 // products overlap the copies of the later bands.
-template <typename T, int KR, bool COH, int MODE, int SP, bool VAR>
+template <typename T, int KR, bool COH, int MODE, int SP>
 __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const T *__restrict__ st1,
                                                        const T *__restrict__ st2, int sx0, int sy0, int px0, int py0,
-                                                       float *prod, uint64_t *bars, unsigned parity, int *err)
+                                                       float *prod, uint64_t *bars, int *err)
 {
     using BS = BlockShape<KR>;
     using SS = StageShape<T, KR>;
@@ -484,10 +474,10 @@ __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const 
     float2 V0n = make_float2(0.f, 0.f);
     if (tid < RW * RW) V0n = fetch_v0_ct<COH, MODE>(a, px0 + rx, py0 + ry);
     auto wait_band = [&](int b) {
-        if (bars && !mbar_wait_bounded(bars + b, parity, 2000000000LL)) {
+        if (bars && !mbar_wait_bounded(bars + b, 0u, 2000000000LL)) {
             // report; the tile's results are then undefined
             if (err) atomicExch(err, 1);
-            mbar_wait_bounded(bars + b, parity, 1000000000LL);
+            mbar_wait_bounded(bars + b, 0u, 1000000000LL);
         }
     };
     unsigned far = 0, bit = 1;  // bit k: the thread's k-th pixel left the staged margin
@@ -503,9 +493,9 @@ __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const 
         }
         if (idx + NT < RW * RW) V0n = fetch_v0_ct<COH, MODE>(a, px0 + rx, py0 + ry);
         float p[5];
-        if (!products_staged_only<T, SP, VAR>(st1, st2, sx0, sy0, a, gx, gy, V0c, p)) far |= bit;
+        if (!products_staged_only<T, SP>(st1, st2, sx0, sy0, a, gx, gy, V0c, p)) far |= bit;
         bit <<= 1;
-        if (VAR && a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) p[0] = p[1] = p[2] = p[3] = p[4] = 0.f;
+        if (a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) p[0] = p[1] = p[2] = p[3] = p[4] = 0.f;
         q[0] = p[0];
         q[PLANE] = p[1];
         q[2 * PLANE] = p[2];
@@ -535,8 +525,8 @@ __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const 
         const int py = UP ? RW - 1 - i / RW : i / RW, px = i - (i / RW) * RW;
         const int gx = px0 + px, gy = py0 + py;
         float p[5];
-        products_interior<T, SP, VAR>(st1, st2, sx0, sy0, a, gx, gy, fetch_v0_ct<COH, MODE>(a, gx, gy), p);
-        if (VAR && a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) p[0] = p[1] = p[2] = p[3] = p[4] = 0.f;
+        products_interior<T, SP>(st1, st2, sx0, sy0, a, gx, gy, fetch_v0_ct<COH, MODE>(a, gx, gy), p);
+        if (a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) p[0] = p[1] = p[2] = p[3] = p[4] = 0.f;
         float *q = prod + py * RWP + px;
         q[0] = p[0];
         q[PLANE] = p[1];
@@ -629,65 +619,41 @@ __device__ __forceinline__ float recip_newton(float d)
 
 // Phase 4 of the forward iteration: the guarded 2x2 solve of pixel (gx, gy)
 // from its window sums S = (Sxx, Sxy, Syy, Sxr, Syr) and the store of V.
-template <bool VAR>
-struct SolveStoreT {
-    template <bool COH>
-    __device__ __forceinline__ void apply(const IterArgs &a, int mode, int gx, int gy, const float (&S)[5]) const
-    {
-        const float sxx = S[0], sxy = S[1], syy = S[2], sxr = S[3], syr = S[4];
-        const float tr = sxx + syy;
-        const float det = sxx * syy - sxy * sxy;
-        float2 V;
-        if (!(tr > a.eps_abs) || det <= a.eps_rel * tr * tr) {
-            V = fetch_v0_rt<COH>(a, mode, gx, gy);
-        } else {
-            const float inv = recip_newton(det);
-            V = make_float2((syy * sxr - sxy * syr) * inv, (sxx * syr - sxy * sxr) * inv);
-            if (VAR && a.inc) {  // increment form: V = V0(m) + H^-1 (Sxr, Syr)
-                const float2 V0 = fetch_v0_rt<COH>(a, mode, gx, gy);
-                V.x += V0.x;
-                V.y += V0.y;
-            }
-        }
-        if (VAR && a.s_out) {  // reverse mode: keep the window sums for the solve adjoint
-            const size_t o = (size_t)gy * a.s_pitch + gx;
-#pragma unroll
-            for (int c = 0; c < 5; ++c) a.s_out[c * a.s_plane + o] = S[c];
-        }
-        if (a.u_out) {
-            if (VAR && a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) V = make_float2(no_vector(), no_vector());
-            a.u_out[(int64_t)gy * a.W + gx] = V.x;
-            a.v_out[(int64_t)gy * a.W + gx] = V.y;
-        } else {
-            a.Vout[(int64_t)gy * a.vpitch + gx] = V;
+template <bool COH>
+__device__ __forceinline__ void solve_store(const IterArgs &a, int mode, int gx, int gy, const float (&S)[5])
+{
+    const float sxx = S[0], sxy = S[1], syy = S[2], sxr = S[3], syr = S[4];
+    const float tr = sxx + syy;
+    const float det = sxx * syy - sxy * sxy;
+    float2 V;
+    if (!(tr > a.eps_abs) || det <= a.eps_rel * tr * tr) {
+        V = fetch_v0_rt<COH>(a, mode, gx, gy);
+    } else {
+        const float inv = recip_newton(det);
+        V = make_float2((syy * sxr - sxy * syr) * inv, (sxx * syr - sxy * sxr) * inv);
+        if (a.inc) {  // increment form: V = V0(m) + H^-1 (Sxr, Syr)
+            const float2 V0 = fetch_v0_rt<COH>(a, mode, gx, gy);
+            V.x += V0.x;
+            V.y += V0.y;
         }
     }
-};
+    if (a.u_out) {
+        if (a.mask && !__ldg(a.mask + (int64_t)gy * a.W + gx)) V = make_float2(no_vector(), no_vector());
+        a.u_out[(int64_t)gy * a.W + gx] = V.x;
+        a.v_out[(int64_t)gy * a.W + gx] = V.y;
+    } else {
+        a.Vout[(int64_t)gy * a.vpitch + gx] = V;
+    }
+}
 
-using SolveStore = SolveStoreT<false>;
-
-// Phases 0-3 of one tile, then epi.apply() per output pixel (phase 4).
-// VAR: the tile honours the estimator variants of a (increment form,
-// Gaussian window); without it the kernel carries no code for them.
+// One tile of the variants' kernels: the estimator variants of a are honoured
+// (increment form, Gaussian window, region mask).
 // TMA staging needs tensor maps tm1, tm2 of the two level images and NBAND
-// mbarriers tma_bars (shared memory): with init_bars the tile initialises
-// them (one tile per CTA), else the caller did and made them visible to the
-// CTA; parity is the phase this tile's copies complete (the number of
-// earlier TMA tiles of the CTA, mod 2).  Returns true when the tile was
-// staged by TMA.
-// Side work a caller may slot into the tile's phases: after_products(tid)
-// runs after phase 1's loop and after_rows(tid) after phase 2's, each before
-// the phase's closing barrier.
-struct NoSide {
-    __device__ __forceinline__ void after_products(int) const {}
-    __device__ __forceinline__ void after_rows(int) const {}
-};
-
-template <typename T, int KR, bool COH, typename Epi = SolveStore, bool VAR = false, typename Side = NoSide>
-__device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, int by, float4 *smem_f4,
-                                           const CUtensorMap *tm1 = nullptr, const CUtensorMap *tm2 = nullptr,
-                                           int *err = nullptr, const Epi &epi = Epi(), uint64_t *tma_bars = nullptr,
-                                           unsigned parity = 0, bool init_bars = false, const Side &side = Side())
+// mbarriers tma_bars (shared memory).
+template <typename T, int KR, bool COH>
+__device__ __forceinline__ void block_tile(const IterArgs &a, int mode, int bx, int by, float4 *smem_f4,
+                                           const CUtensorMap *tm1, const CUtensorMap *tm2, int *err,
+                                           uint64_t *tma_bars)
 {
     using BS = BlockShape<KR>;
     using SS = StageShape<T, KR>;
@@ -722,11 +688,7 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
     if (tm1 != nullptr && tma_bars != nullptr && interior && (smem_u32(stage) & 127u) == 0) {
         // NBAND bands of SHB rows per frame, band b of both frames on barrier b
         if (tid == 0) {
-            if (init_bars)
-                for (int b = 0; b < NBAND; ++b) mbar_init(&tma_bars[b], 1);
-            // order earlier generic-proxy accesses of the buffer (a previous
-            // tile of this CTA) before the copies
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_init_n<NBAND>(tma_bars);
             for (int k = 0; k < NBAND; ++k) {
                 const int b = UP ? NBAND - 1 - k : k;  // the band phase 1 needs first, first
                 mbar_expect_tx(&tma_bars[b], (unsigned)(2 * SHB * SP * sizeof(T)));
@@ -734,7 +696,7 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
                 tma_load_2d(stage + STG + b * SHB * SP, tm2, sx0, sy0 + b * SHB, &tma_bars[b]);
             }
         }
-        if (init_bars) __syncthreads();  // barriers initialised before anyone waits on them
+        __syncthreads();  // barriers initialised before anyone waits on them
         bars = tma_bars;
     } else {
         for (int t = tid; t < 2 * SH * NV; t += NT) {
@@ -763,16 +725,16 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
     if (interior) {
         const T *st2 = stage + STG;
         if (mode == V0_SAME)
-            products_tile_interior<T, KR, COH, V0_SAME, SP, VAR>(a, stage, st2, sx0, sy0, px0, py0, prod, bars, parity,
+            products_tile_interior<T, KR, COH, V0_SAME, SP>(a, stage, st2, sx0, sy0, px0, py0, prod, bars,
                                                            err);
         else if (mode == V0_UP)
-            products_tile_interior<T, KR, COH, V0_UP, SP, VAR>(a, stage, st2, sx0, sy0, px0, py0, prod, bars, parity, err);
+            products_tile_interior<T, KR, COH, V0_UP, SP>(a, stage, st2, sx0, sy0, px0, py0, prod, bars, err);
         else
-            products_tile_interior<T, KR, COH, V0_ZERO, SP, VAR>(a, stage, st2, sx0, sy0, px0, py0, prod, bars, parity,
+            products_tile_interior<T, KR, COH, V0_ZERO, SP>(a, stage, st2, sx0, sy0, px0, py0, prod, bars,
                                                            err);
         // every band has landed before the CTA can finish (no copy in flight at exit)
         if (bars && tid == 0)
-            for (int b = 0; b < NBAND; ++b) mbar_wait_bounded(&bars[b], parity, 1000000000LL);
+            for (int b = 0; b < NBAND; ++b) mbar_wait_bounded(&bars[b], 0u, 1000000000LL);
     } else {
         // index step in rows and columns (rows in the order of RowOrder)
         constexpr int DX = NT % RW, DY = UP ? -(NT / RW) : NT / RW, DW = UP ? -1 : 1;
@@ -791,7 +753,7 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
                 V0n = fetch_v0_rt<COH>(a, mode, px0 + nrx, py0 + nry);
             float p[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
             if (gx > kBlockReach && gx < W - kBlockReach - 2 && gy > kBlockReach && gy < H - kBlockReach - 2) {
-                products_interior<T, SP, VAR>(stage, stage + STG, sx0, sy0, a, gx, gy, V0c, p);
+                products_interior<T, SP>(stage, stage + STG, sx0, sy0, a, gx, gy, V0c, p);
             } else if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
                 const float2 V0 = V0c;
                 const float hx = 0.5f * V0.x, hy = 0.5f * V0.y;
@@ -799,7 +761,7 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
                 const Sample s2 = sample_staged<T, SP>(stage + STG, sx0, sy0, P2, H, W, pitch, gx, gy, hx, hy);
                 const float Gx = 0.5f * (s1.gx + s2.gx), Gy = 0.5f * (s1.gy + s2.gy);
                 const float It = s2.val - s1.val;
-                const float r = (VAR && a.inc) ? -It : Gx * V0.x + Gy * V0.y - It;
+                const float r = a.inc ? -It : Gx * V0.x + Gy * V0.y - It;
                 p[0] = Gx * Gx;
                 p[1] = Gx * Gy;
                 p[2] = Gy * Gy;
@@ -807,7 +769,7 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
                 p[4] = Gy * r;
             }
             // a masked pixel leaves the window sums
-            if (VAR && a.mask && gy >= 0 && gy < H && gx >= 0 && gx < W && !__ldg(a.mask + (int64_t)gy * W + gx))
+            if (a.mask && gy >= 0 && gy < H && gx >= 0 && gx < W && !__ldg(a.mask + (int64_t)gy * W + gx))
                 p[0] = p[1] = p[2] = p[3] = p[4] = 0.f;
             float *q = prod + ry * RWP + rx;
             q[0] = p[0];
@@ -819,12 +781,11 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
             rx = nrx;
         }
     }
-    side.after_products(tid);
     __syncthreads();
 
     // phase 2: horizontal window sums, one (row, channel) per thread
     // (weighted sums with the Gaussian window)
-    if (VAR && a.gauss) {
+    if (a.gauss) {
         for (int t = tid; t < 5 * RW; t += NT) {
             const int c = t / RW, row = t - c * RW;
             window_wsums_inplace<R, TS>(prod + c * PLANE + row * RWP, 1, a.wg);
@@ -835,11 +796,10 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
             window_sums_inplace<R, TS>(prod + c * PLANE + row * RWP, 1);
         }
     }
-    side.after_rows(tid);
     __syncthreads();
 
     // phase 3: vertical window sums, one (column, channel) per thread
-    if (VAR && a.gauss) {
+    if (a.gauss) {
         for (int t = tid; t < 5 * TS; t += NT) {
             const int c = t / TS, col = t - c * TS;
             window_wsums_inplace<R, TS>(prod + c * PLANE + col, RWP, a.wg);
@@ -852,47 +812,30 @@ __device__ __forceinline__ bool block_tile(const IterArgs &a, int mode, int bx, 
     }
     __syncthreads();
 
-    // phase 4: per output pixel, the epilogue (guarded solve and store)
+    // phase 4: per output pixel, the guarded solve and store
     for (int idx = tid; idx < TS * TS; idx += NT) {
         const int oy = idx / TS, ox = idx - oy * TS;
         const int gy = ty0 + oy, gx = tx0 + ox;
         if (gy >= H || gx >= W) continue;
         const float *q = prod + oy * RWP + ox;
         const float S[5] = {q[0], q[PLANE], q[2 * PLANE], q[3 * PLANE], q[4 * PLANE]};
-        epi.template apply<COH>(a, mode, gx, gy, S);
-    }
-    return bars != nullptr;
-}
-
-// One tile per CTA; blockIdx.z selects the pair.  VAR: estimator variants.
-template <typename T, int KR, bool VAR>
-__global__ void __launch_bounds__(BlockShape<KR>::NT, BlockShape<KR>::MINB) k_iter_block(const __grid_constant__ BlockParams prm)
-{
-    extern __shared__ __align__(128) float4 smem_f4[];
-    __shared__ __align__(8) uint64_t s_bar[StageShape<T, KR>::NBAND];
-    const int z = blockIdx.z;
-    if (prm.use_tma) {
-        block_tile<T, KR, false, SolveStoreT<VAR>, VAR>(prm.a[z], prm.mode, blockIdx.x, blockIdx.y + prm.by0, smem_f4,
-                                                        &prm.tm[z][0], &prm.tm[z][1], prm.err, SolveStoreT<VAR>(),
-                                                        s_bar, 0u, true);
-    } else {
-        block_tile<T, KR, false, SolveStoreT<VAR>, VAR>(prm.a[z], prm.mode, blockIdx.x, blockIdx.y + prm.by0,
-                                                        smem_f4);
+        solve_store<COH>(a, mode, gx, gy, S);
     }
 }
 
 // ---------------------------------------------------------------------------
-// Persistent batched launch: many pairs of unequal size, all (level,
-// iteration) stages, in one launch.  Work units (stage, pair, tile) are
-// handed out in the order of a schedule built on the host; a unit of stage
-// s waits until every tile of stage s-1 of its pair is done (a per-(stage,
-// pair) counter).  Units are claimed in schedule order by resident CTAs,
-// each CTA one unit ahead of the one it runs; a unit depends only on
-// earlier units, so the earliest unfinished unit is always being run by its
-// CTA (any unit before it in that CTA is finished) and the launch cannot
-// stall on itself.  The wait is bounded
-// by an iteration count and a %globaltimer deadline; on expiry the CTA
-// records an error word and leaves, and the host reports OFV_ERR_TIMEOUT.
+// Batched launch: many pairs of unequal size, all (level, iteration) stages,
+// in one launch of one CTA per work unit (stage, pair, tile).  A CTA claims
+// the next unit of a schedule built on the host when it starts; a unit of
+// stage s waits until every tile of stage s-1 of its pair is done (a
+// per-(stage, pair) counter).  Units are claimed in schedule order by CTAs
+// that are resident, and a unit depends only on earlier units, so the
+// earliest unfinished unit is always running and the launch cannot stall on
+// itself, in whatever order the CTAs start.  The wait is bounded by an
+// iteration count and a %globaltimer deadline; on expiry the CTA records an
+// error word and leaves, and the host reports OFV_ERR_TIMEOUT.
+// (Resident CTAs looping over units kept the walk's tile-invariant addresses
+// across tiles and spilled 448 bytes of stack.)
 // ---------------------------------------------------------------------------
 struct BatchPair {
     const void *P1[16], *P2[16];  // level images of the two frames
@@ -920,156 +863,21 @@ struct QueueParams {
     int *host_err;             // mapped host word: 1 + the unit whose wait expired, or null
 };
 
-__device__ __forceinline__ int ld_acquire(const int *p)
-{
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// The persistent kernel's side work (see NoSide): thread 0 publishes the
-// unit it claimed for after this tile, and a thread with no line in the
-// row pass reads that unit's descriptor and looks once whether its
-// dependency is already complete, so the next unit starts without those
-// round trips.
-struct QueueSide {
-    const QueueParams *q;
-    int next;          // thread 0: the claimed next unit
-    int side_tid;      // the thread that prefetches
-    int *s_next;
-    int4 *s_dec;       // prefetched descriptor
-    int *s_dec_unit;   // its unit (-1: none)
-    int *s_dec_ok;     // 1: its dependency was seen complete
-    __device__ __forceinline__ void after_products(int tid) const
-    {
-        if (tid == 0) *s_next = next;
-    }
-    __device__ __forceinline__ void after_rows(int tid) const
-    {
-        if (tid != side_tid) return;
-        const int n = *s_next;
-        if (n >= q->total_units) return;
-        const int4 d = __ldg(q->unit_desc + n);
-        *s_dec_ok = d.x == 0 || ld_acquire(q->done + (d.x - 1) * q->npairs + d.y) >= d.w;
-        *s_dec = d;
-        *s_dec_unit = n;
-    }
+// Host launchers, explicitly instantiated per level storage type T and kind
+// of iteration in k_block_{f32,f16,bf16}.cu (ITER_BOX) and
+// k_block_var_{f32,f16,bf16}.cu (ITER_KEEP and ITER_VAR).
+// shape: the tile shape v (ITER_KEEP and ITER_VAR have the default shape
+// only; the batched launch has no ITER_KEEP)
+enum IterKind : int {
+    ITER_BOX = 0,   // uniform box window (k_walk.cuh)
+    ITER_KEEP = 1,  // the same, keeping the window sums for the reverse mode
+    ITER_VAR = 2    // estimator variants: Gaussian window, increment form, region mask
 };
-
-template <typename T, int KR, bool VAR>
-__global__ void __launch_bounds__(BlockShape<KR>::NT, BlockShape<KR>::MINB) k_iter_queue(const __grid_constant__ QueueParams q)
-{
-    constexpr int TS = BlockShape<KR>::TS;
-    extern __shared__ __align__(128) float4 smem_f4[];
-    __shared__ int s_unit, s_fail, s_next, s_dec_unit, s_dec_ok;
-    __shared__ int4 s_dec;
-    __shared__ __align__(8) uint64_t s_bar[StageShape<T, KR>::NBAND];
-    const int S = q.L * q.IT;
-    unsigned tma_uses = 0;  // TMA-staged tiles of this CTA so far
-    if (q.tmaps && threadIdx.x == 0)
-        for (int b = 0; b < StageShape<T, KR>::NBAND; ++b) mbar_init(&s_bar[b], 1);  // visible after the loop's first barrier
-    if (threadIdx.x == 0) {
-        s_unit = atomicAdd(q.head, 1);
-        s_fail = 0;
-        s_dec_unit = -1;
-    }
-    __syncthreads();
-    // thread 0: the (stage, pair) whose previous stage it last saw complete
-    int checked = -1;
-    for (;;) {
-        const int unit = s_unit;
-        if (unit >= q.total_units) break;
-        // the unit's descriptor, prefetched during the previous tile when
-        // this CTA ran one
-        const bool pre = s_dec_unit == unit;
-        const int4 d = pre ? s_dec : __ldg(q.unit_desc + unit);
-        const bool pre_ok = pre && s_dec_ok;
-        const int s = d.x, p = d.y, tile = d.z, need = d.w;
-        const int key = s * q.npairs + p;
-        const BatchPair &bp = q.pairs[p];
-        const int l = q.L - 1 - s / q.IT, t = s % q.IT;
-        // the next unit is claimed now and read after this tile, so the
-        // claim's round trip overlaps the tile's work
-        int next = 0;
-        if (threadIdx.x == 0) next = atomicAdd(q.head, 1);
-        if (s > 0 && threadIdx.x == 0 && !pre_ok && checked != key) {
-            const int *cnt = q.done + (s - 1) * q.npairs + p;
-            const long long t0 = global_ns();
-            int spins = 0;
-            while (ld_acquire(cnt) < need) {
-                if (++spins > q.spin_limit || global_ns() - t0 > q.timeout_ns) {
-                    atomicCAS(q.error, 0, 1 + unit);
-                    if (q.host_err) *reinterpret_cast<volatile int *>(q.host_err) = 1 + unit;
-                    s_fail = 1;
-                    break;
-                }
-                __nanosleep(128);
-            }
-            checked = key;
-        }
-        __syncthreads();
-        if (s_fail) break;
-        IterArgs a = {};
-        a.P1 = bp.P1[l];
-        a.P2 = bp.P2[l];
-        a.H = bp.H[l];
-        a.W = bp.W[l];
-        a.pitch = bp.pitch[l];
-        a.vpitch = bp.vpitch;
-        a.vcpitch = bp.vpitch;
-        a.kr = q.kr;
-        a.eps_rel = q.eps_rel;
-        a.eps_abs = q.eps_abs;
-        if (VAR) {
-            a.inc = q.inc;
-            a.gauss = q.gauss;
-#pragma unroll
-            for (int d = 0; d <= kBlockMaxKR; ++d) a.wg[d] = q.wg[d];
-        }
-        int mode = V0_ZERO;
-        if (s > 0 && t == 0) {
-            mode = V0_UP;
-            a.Vc = bp.vb[(s - 1) & 1];
-            a.Hc = bp.H[l + 1];
-            a.Wc = bp.W[l + 1];
-        } else if (s > 0) {
-            mode = V0_SAME;
-            a.V0 = bp.vb[(s - 1) & 1];
-        }
-        if (s == S - 1) {
-            a.u_out = bp.u;
-            a.v_out = bp.v;
-        } else {
-            a.Vout = bp.vb[s & 1];
-        }
-        const int ntx = (a.W + TS - 1) / TS;
-        const CUtensorMap *tm = q.tmaps ? q.tmaps + ((size_t)p * 16 + l) * 2 : nullptr;
-        const QueueSide side{&q, next, BlockShape<KR>::NT - 1, &s_next, &s_dec, &s_dec_unit, &s_dec_ok};
-        if (block_tile<T, KR, true, SolveStoreT<VAR>, VAR, QueueSide>(a, mode, tile % ntx, tile / ntx, smem_f4, tm,
-                                                                      tm ? tm + 1 : nullptr, q.tma_err,
-                                                                      SolveStoreT<VAR>(), q.tmaps ? s_bar : nullptr,
-                                                                      tma_uses & 1u, false, side))
-            ++tma_uses;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            atomicAdd(q.done + key, 1);
-            s_unit = next;
-        }
-        __syncthreads();
-    }
-}
-
-// Host launchers, explicitly instantiated per level storage type T and
-// variant flag VAR in k_block_{f32,f16,bf16}.cu (VAR = false, plus the
-// reverse-mode stage kernel) and k_block_var_{f32,f16,bf16}.cu (VAR = true).
-// shape: the tile shape v (the estimator variants, VAR = true, have the
-// default shape only)
-template <typename T, bool VAR>
-cudaError_t launch_block_t(const BlockParams &p, int kr, int npairs, cudaStream_t s, int nrows = 0, int shape = 0);
-template <typename T, bool VAR>
-cudaError_t launch_queue_t(const QueueParams &q, int kr, int ctas, cudaStream_t s, int shape = 0);
-template <typename T, bool VAR>
+template <typename T, int KIND>
+cudaError_t launch_block_t(const BlockParams &p, int kr, int npairs, cudaStream_t s, int shape = 0);
+template <typename T, int KIND>
+cudaError_t launch_queue_t(const QueueParams &q, int kr, cudaStream_t s, int shape = 0);
+template <typename T, int KIND>
 int queue_occupancy_t(int kr, int shape = 0);
 
 // Output tile edge of the block kernel for radius kr and tile shape v.

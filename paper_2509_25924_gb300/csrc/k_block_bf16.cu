@@ -1,10 +1,10 @@
-// Block-tiled iteration kernels for __nv_bfloat16 level storage, window radii 1..10:
-// the estimator as read from Sec. 2 (no variant code) and the persistent
-// batched form.
+// Iteration kernels for __nv_bfloat16 level storage, window radii 1..10: the
+// estimator as read from Sec. 2, one tile per CTA and batched.
 #include "k_block_inst.cuh"
 
 namespace ofv {
 
-OFV_INSTANTIATE_BLOCK_LAUNCHERS(__nv_bfloat16, false)
+OFV_INSTANTIATE_BLOCK(__nv_bfloat16, ITER_BOX)
+OFV_INSTANTIATE_QUEUE(__nv_bfloat16, ITER_BOX)
 
 }  // namespace ofv

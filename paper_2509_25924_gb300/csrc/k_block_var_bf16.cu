@@ -1,9 +1,12 @@
-// Block-tiled iteration kernels for __nv_bfloat16 level storage, window radii 1..10,
-// with the estimator variants (increment form, Gaussian window).
+// Iteration kernels for __nv_bfloat16 level storage, window radii 1..10, with the
+// estimator variants (increment form, Gaussian window, region mask), and the
+// form that keeps the window sums for the reverse mode.
 #include "k_block_inst.cuh"
 
 namespace ofv {
 
-OFV_INSTANTIATE_BLOCK_LAUNCHERS(__nv_bfloat16, true)
+OFV_INSTANTIATE_BLOCK(__nv_bfloat16, ITER_KEEP)
+OFV_INSTANTIATE_BLOCK(__nv_bfloat16, ITER_VAR)
+OFV_INSTANTIATE_QUEUE(__nv_bfloat16, ITER_VAR)
 
 }  // namespace ofv

@@ -1,7 +1,6 @@
-// Batched entry point: many image pairs of unequal size in one persistent
-// launch (a work queue of (stage, pair, tile) units), with an autotuner that
-// picks the unit schedule and the number of persistent CTAs per batch
-// signature.
+// Batched entry point: many image pairs of unequal size in one launch (a
+// work queue of (stage, pair, tile) units, one CTA each), with an autotuner
+// that picks the unit schedule and the tile shape per batch signature.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -16,15 +15,15 @@
 #include "ofv_handle.h"
 
 namespace ofv {
-#define OFV_EXTERN_QUEUE(T, VAR)                                                                   \
-    extern template cudaError_t launch_queue_t<T, VAR>(const QueueParams &, int, int, cudaStream_t, int); \
-    extern template int queue_occupancy_t<T, VAR>(int, int);
-OFV_EXTERN_QUEUE(float, false)
-OFV_EXTERN_QUEUE(float, true)
-OFV_EXTERN_QUEUE(__half, false)
-OFV_EXTERN_QUEUE(__half, true)
-OFV_EXTERN_QUEUE(__nv_bfloat16, false)
-OFV_EXTERN_QUEUE(__nv_bfloat16, true)
+#define OFV_EXTERN_QUEUE(T, KIND)                                                                   \
+    extern template cudaError_t launch_queue_t<T, KIND>(const QueueParams &, int, cudaStream_t, int); \
+    extern template int queue_occupancy_t<T, KIND>(int, int);
+OFV_EXTERN_QUEUE(float, ITER_BOX)
+OFV_EXTERN_QUEUE(float, ITER_VAR)
+OFV_EXTERN_QUEUE(__half, ITER_BOX)
+OFV_EXTERN_QUEUE(__half, ITER_VAR)
+OFV_EXTERN_QUEUE(__nv_bfloat16, ITER_BOX)
+OFV_EXTERN_QUEUE(__nv_bfloat16, ITER_VAR)
 #undef OFV_EXTERN_QUEUE
 }  // namespace ofv
 
@@ -38,17 +37,17 @@ constexpr int kWaitSpinLimit = 200000000;
 // The kernels with variant code run only when a variant is on.
 // shape: the block kernel's tile shape (0 default, 1 alternative; the
 // variant kernels have the default only).
-cudaError_t launch_queue(int store, const QueueParams &q, int kr, int ctas, cudaStream_t s, int shape)
+cudaError_t launch_queue(int store, const QueueParams &q, int kr, cudaStream_t s, int shape)
 {
     const bool var = q.inc || q.gauss;
     switch (store) {
-    case OFV_STORE_F16: return var ? launch_queue_t<__half, true>(q, kr, ctas, s, shape)
-                                   : launch_queue_t<__half, false>(q, kr, ctas, s, shape);
-    case OFV_STORE_BF16: return var ? launch_queue_t<__nv_bfloat16, true>(q, kr, ctas, s, shape)
-                                    : launch_queue_t<__nv_bfloat16, false>(q, kr, ctas, s, shape);
+    case OFV_STORE_F16: return var ? launch_queue_t<__half, ITER_VAR>(q, kr, s, shape)
+                                   : launch_queue_t<__half, ITER_BOX>(q, kr, s, shape);
+    case OFV_STORE_BF16: return var ? launch_queue_t<__nv_bfloat16, ITER_VAR>(q, kr, s, shape)
+                                    : launch_queue_t<__nv_bfloat16, ITER_BOX>(q, kr, s, shape);
     default:
-        return var ? launch_queue_t<float, true>(q, kr, ctas, s, shape)
-                   : launch_queue_t<float, false>(q, kr, ctas, s, shape);
+        return var ? launch_queue_t<float, ITER_VAR>(q, kr, s, shape)
+                   : launch_queue_t<float, ITER_BOX>(q, kr, s, shape);
     }
 }
 
@@ -56,11 +55,11 @@ int queue_occupancy(int store, int kr, bool var, int shape)
 {
     switch (store) {
     case OFV_STORE_F16:
-        return var ? queue_occupancy_t<__half, true>(kr, shape) : queue_occupancy_t<__half, false>(kr, shape);
+        return var ? queue_occupancy_t<__half, ITER_VAR>(kr, shape) : queue_occupancy_t<__half, ITER_BOX>(kr, shape);
     case OFV_STORE_BF16:
-        return var ? queue_occupancy_t<__nv_bfloat16, true>(kr, shape)
-                   : queue_occupancy_t<__nv_bfloat16, false>(kr, shape);
-    default: return var ? queue_occupancy_t<float, true>(kr, shape) : queue_occupancy_t<float, false>(kr, shape);
+        return var ? queue_occupancy_t<__nv_bfloat16, ITER_VAR>(kr, shape)
+                   : queue_occupancy_t<__nv_bfloat16, ITER_BOX>(kr, shape);
+    default: return var ? queue_occupancy_t<float, ITER_VAR>(kr, shape) : queue_occupancy_t<float, ITER_BOX>(kr, shape);
     }
 }
 
@@ -137,10 +136,11 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
             return fail_msg(OFV_ERR_SHAPE, "ofv_compute_batched: pair %d (%dx%d): coarsest level below %d", i, q.H,
                             q.W, minsz);
         for (int t : shapes) {
-            const int TS = block_tile_size(KR, t);
+            const int tw = var ? block_tile_size(KR, t) : walk_tile_w(KR, t);
+            const int th = var ? block_tile_size(KR, t) : walk_tile_h(KR, t);
             for (int s = 0; s < S; ++s) {
                 const int l = L - 1 - s / IT;
-                tiles[t][i][s] = ((Ws[i][l] + TS - 1) / TS) * ((Hs[i][l] + TS - 1) / TS);
+                tiles[t][i][s] = ((Ws[i][l] + tw - 1) / tw) * ((Hs[i][l] + th - 1) / th);
             }
         }
     }
@@ -327,7 +327,7 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
                 for (int l = 0; l < L && ok; ++l)
                     for (int f = 0; f < 2 && ok; ++f)
                         ok = encode_block_map(&maps[((size_t)i * 16 + l) * 2 + f], lvl(i, f, l), Ws[i][l], Hs[i][l],
-                                              pitch_for(Ws[i][l]), p.storage, KR, shape);
+                                              pitch_for(Ws[i][l]), p.storage, KR, shape, variant_of(p));
             if (!ok) return false;
             if (h->batch_maps.size() > 64) h->batch_maps.clear();
             mit = h->batch_maps.emplace(k, std::move(maps)).first;
@@ -348,8 +348,7 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
         return true;
     };
 
-    int dev = h->device, sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int dev = h->device;
 
     // batch signature for the autotuner
     std::vector<std::pair<int, int>> sizes;
@@ -368,8 +367,7 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
         for (int t : shapes) {
             const int occ = std::max(1, queue_occupancy(p.storage, KR, var, t));
             for (int sch : {0, 8})
-                for (int c : {occ, occ - 1})
-                    if (c >= 1 && (sch == 0 || sch < n)) cands.push_back(BatchTune{sch, c, t, 0.0});
+                if (sch == 0 || sch < n) cands.push_back(BatchTune{sch, occ, t, 0.0});
         }
     } else {
         cands.push_back(it->second);
@@ -413,7 +411,7 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
         cudaEventCreate(&ev.b);
     }
     std::vector<int4> desc;
-    // one persistent launch of candidate c (timed while tuning)
+    // one launch of candidate c (timed while tuning)
     auto run = [&](size_t c, bool timed) -> ofv_status {
         const int shape = cands[c].shape;
         const bool use_tma = ensure_maps(shape);
@@ -430,10 +428,9 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
         }
         if (e == cudaSuccess) e = cudaMemsetAsync(q.done, 0, sizeof(int) * (maxgroups + 2), cs);
         if (e != cudaSuccess) return cuda_fail_msg(e, "ofv_compute_batched: uploading the schedule");
-        const int ctas = std::min(sms * cands[c].ctas_per_sm, std::max(1, q.total_units));
         if (timed) cudaEventRecord(ev.a, cs);
-        e = launch_queue(p.storage, q, KR, ctas, cs, shape);
-        if (e != cudaSuccess) return cuda_fail_msg(e, "ofv_compute_batched: persistent launch");
+        e = launch_queue(p.storage, q, KR, cs, shape);
+        if (e != cudaSuccess) return cuda_fail_msg(e, "ofv_compute_batched: launch");
         if (timed) {
             cudaEventRecord(ev.b, cs);
             e = cudaEventSynchronize(ev.b);
@@ -455,9 +452,8 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
     }
     if (tuning) {
         h->tune[key] = cands[best];
-        // Candidates of one tile shape compute the same fields; another shape
-        // sums the windows in another order.  The fields left in place must be
-        // the chosen configuration's, as in every later call of this signature.
+        // Every candidate computes the same fields.  The tensor maps left in
+        // the arena must be the chosen shape's, as recording expects.
         if (cands[best].shape != cands.back().shape) {
             const ofv_status st = run((size_t)best, false);
             if (st != OFV_OK) return st;
@@ -549,7 +545,7 @@ ofv_status ofv_batch_tuning(const ofv_handle *h, int *schedule, int *ctas_per_sm
     return OFV_OK;
 }
 
-// A persistent launch whose one work unit waits on a counter that nothing
+// A batched launch whose one work unit waits on a counter that nothing
 // increments; the wait must expire after about timeout_us and leave the
 // error word set (1 + the unit) for the host, without a fault or a hang.
 ofv_status ofv_queue_selftest(int timeout_us, int *error_word)
@@ -591,7 +587,7 @@ ofv_status ofv_queue_selftest(int timeout_us, int *error_word)
     if (e == cudaSuccess) {
         *hw = 0;
         q.host_err = hw_d;
-        e = launch_queue(OFV_STORE_F32, q, 4, 1, nullptr, 0);
+        e = launch_queue(OFV_STORE_F32, q, 4, nullptr, 0);
     }
     int err = 0;
     if (e == cudaSuccess) e = cudaMemcpy(&err, q.error, sizeof(int), cudaMemcpyDeviceToHost);

@@ -168,19 +168,19 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder_impl()
 }
 
 // Tensor maps of the level images for the block kernel's staged box (see
-// encode_block_map).  Levels smaller than the box never have an interior
-// tile and keep cp.async.
+// encode_block_map).  A level whose maps cannot be encoded keeps cp.async.
 void encode_tensor_maps(ofv_handle *h)
 {
     int cols = 0, rows = 0;
-    block_stage_box(h->p.storage, h->p.kernel_radius, &cols, &rows, tile_shape_of(h->p));
+    const bool var = variant_of(h->p);
+    block_stage_box(h->p.storage, h->p.kernel_radius, &cols, &rows, tile_shape_of(h->p), var);
     for (int l = 0; l < h->L; ++l) {
         h->tma_ok[l] = 0;
-        if (cols < 1 || h->Ws[l] < cols || h->Hs[l] < rows) continue;
+        if (cols < 1) continue;
         bool ok = true;
         for (int f = 0; f < h->nslots && ok; ++f)
             ok = encode_block_map(&h->tmap[f][l], h->lvl[f][l], h->Ws[l], h->Hs[l], h->pitch[l], h->p.storage,
-                                  h->p.kernel_radius, tile_shape_of(h->p));
+                                  h->p.kernel_radius, tile_shape_of(h->p), var);
         h->tma_ok[l] = ok ? 1 : 0;
     }
 }
@@ -511,11 +511,11 @@ ofv_status handle_pyramids(ofv_handle *h, const void *const *frames, const int *
 // stride pitch elements) with the block kernel's TMA box for radius kr; no
 // swizzle, out-of-bounds fill unused (only boxes inside the image are
 // copied).  False when the encoder is unavailable or refuses.
-bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch, int store, int kr, int shape)
+bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch, int store, int kr, int shape, bool var)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder_impl();
     int cols = 0, rows = 0;
-    block_stage_box(store, kr, &cols, &rows, shape);
+    block_stage_box(store, kr, &cols, &rows, shape, var);
     if (!enc || cols < 1) return false;
     const CUtensorMapDataType dt = store == OFV_STORE_F16    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                    : store == OFV_STORE_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16

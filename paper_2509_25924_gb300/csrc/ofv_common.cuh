@@ -87,15 +87,17 @@ cudaError_t launch_iter_fused(const IterArgs &a, int store, int mode, cudaStream
 bool block_supports(int kr);
 // The forward solve's reciprocal of x[0..n-1] into y (device arrays), for tests.
 cudaError_t launch_recip(const float *x, float *y, int n, cudaStream_t s);
-// by0, nby: tile rows by0 .. by0+nby-1 only (nby 0: to the bottom of the level).
+// row0, nrows: output rows row0 .. row0+nrows-1 only, row0 a multiple of the
+// tile edge (nrows 0: to the bottom of the level).
 // shape: the tile shape (0 default, 1 the alternative; the estimator
 // variants run the default shape).
 cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode, cudaStream_t s,
-                              const CUtensorMap *const *tm = nullptr, int *err = nullptr, int by0 = 0, int nby = 0,
+                              const CUtensorMap *const *tm = nullptr, int *err = nullptr, int row0 = 0, int nrows = 0,
                               int shape = 0);
-// TMA box of the block kernel's staging (columns, rows of one band) for this
-// storage, radius and tile shape.
-void block_stage_box(int store, int kr, int *cols, int *rows, int shape = 0);
+// TMA box of the iteration kernels' staging (columns, rows of one band) for
+// this storage, radius and tile shape; var: of the estimator variants'
+// kernels (Gaussian window, increment form).
+void block_stage_box(int store, int kr, int *cols, int *rows, int shape = 0, bool var = false);
 
 struct PlainBufs {
     float *prod;  // 5 planes, each H x pitch floats

@@ -28,9 +28,9 @@ struct ProfRec {
 // signature (sizes and parameters).
 struct BatchTune {
     int schedule;     // 0: stage-major over all pairs, else pairs in groups of this many
-    int ctas_per_sm;  // persistent CTAs per SM
+    int ctas_per_sm;  // resident CTAs per SM
     int shape;        // block kernel tile shape (0 default, 1 alternative)
-    double ms;        // measured duration of the persistent launch
+    double ms;        // measured duration of the launch
 };
 
 // Record a failure for ofv_last_error() (thread-local) and return st.
@@ -131,7 +131,10 @@ cudaError_t dev_alloc(void **p, size_t bytes);
 // Steps 1-2 into the handle's pyramid slots (defined with the C ABI).
 ofv_status handle_pyramids(ofv_handle *h, const void *const *frames, const int *slots, int nf, cudaStream_t s);
 // Tensor map of a level image with the block kernel's TMA box.
-bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch, int store, int kr, int shape = 0);
+bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch, int store, int kr, int shape = 0,
+                      bool var = false);
+// The estimator variants whose kernels a handle runs throughout.
+inline bool variant_of(const ofv_params &p) { return p.window == OFV_WINDOW_GAUSS || p.increment_form; }
 // Tile shape of the block kernel that params select: 0 (default) or 1 (the
 // alternative edge), -1 when tile_edge is not one of the radius's edges on
 // the fused block path.  The Gaussian window and the increment form run the

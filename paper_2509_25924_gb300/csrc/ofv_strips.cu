@@ -281,7 +281,6 @@ extern "C" ofv_status ofv_compute_strips(ofv_handle *h, int nstrips, int max_dis
 
     // steps 3-6: coarse to fine, every strip's tiles, then the halo copies
     const int shape = tile_shape_of(p);
-    const int ts = block_tile_size(p.kernel_radius, shape);
     int cur = 0;
     for (int l = L - 1; l >= 0; --l) {
         for (int t = 0; t < IT; ++t) {
@@ -317,8 +316,8 @@ extern "C" ofv_status ofv_compute_strips(ofv_handle *h, int nstrips, int max_dis
                 } else {
                     a.Vout = sb[d].fld[nxt];
                 }
-                if ((e = launch_iter_block(&a, 1, p.storage, mode, s, nullptr, nullptr, own.a / ts,
-                                           (own.b - own.a + ts - 1) / ts, shape)) != cudaSuccess)
+                if ((e = launch_iter_block(&a, 1, p.storage, mode, s, nullptr, nullptr, own.a, own.b - own.a,
+                                           shape)) != cudaSuccess)
                     return launch_fail("strips: iteration");
             }
             if (last) break;
