@@ -21,6 +21,7 @@
 
 #include "iter_math.cuh"
 #include "k_bw_block.cuh"
+#include "k_bw_walk.cuh"
 #include "ofv_handle.h"
 
 namespace ofv {
@@ -216,52 +217,26 @@ __global__ void k_bw_samples(IterArgs a, Planes5 gprod, float2 *gV0, float *gP1,
     samples_adjoint_pixel<T>(a, gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
 }
 
-// A 32 x 32 tile of pixels per CTA.  The image-gradient scatter lands in a
-// shared-memory window around the tile (margin REACH + 2, which holds every
-// tap of a warp up to REACH px) and reaches global memory once per window
-// element; taps outside the window (larger warps) go to global memory
-// directly.  Windows of neighbouring tiles overlap, so the final adds are
-// atomic too.
-constexpr int kSampTS = 32, kSampM = kBlockReach + 2, kSampWW = kSampTS + 2 * kSampM;
-
-struct ScatterWindow {
-    float (*win)[kSampWW + 1];
-    float *g;
-    int pitch, wx0, wy0;
-    __device__ __forceinline__ void operator()(int y, int x, float v) const
-    {
-        const int r = y - wy0, c = x - wx0;
-        if ((unsigned)r < (unsigned)kSampWW && (unsigned)c < (unsigned)kSampWW)
-            atomicAdd(&win[r][c], v);
-        else
-            atomicAdd(g + (int64_t)y * pitch + x, v);
-    }
-};
-
+// The walk's pixels that need the general form: a call, which keeps the
+// walk's registers apart from it.
 template <typename T>
-__global__ void __launch_bounds__(256) k_bw_samples_tile(IterArgs a, Planes5 gprod, float2 *gV0, float *gP1,
-                                                         float *gP2, int gpitch)
+__device__ __noinline__ void samples_adjoint_general(const IterArgs *a, const Planes5 *gprod, float2 *gV0, int x, int y,
+                                                     float *gP1, float *gP2, int gpitch)
 {
-    __shared__ float acc[2][kSampWW][kSampWW + 1];
-    const int tid = threadIdx.x;
-    const int tx0 = blockIdx.x * kSampTS, ty0 = blockIdx.y * kSampTS;
-    const int wx0 = tx0 - kSampM, wy0 = ty0 - kSampM;
-    float *flat = &acc[0][0][0];
-    for (int i = tid; i < 2 * kSampWW * (kSampWW + 1); i += 256) flat[i] = 0.f;
-    __syncthreads();
-    const ScatterWindow s1{acc[0], gP1, gpitch, wx0, wy0}, s2{acc[1], gP2, gpitch, wx0, wy0};
-    for (int i = tid; i < kSampTS * kSampTS; i += 256) {
-        const int y = ty0 + i / kSampTS, x = tx0 + i % kSampTS;
-        if (y < a.H && x < a.W) samples_adjoint_pixel<T>(a, gprod, gV0, x, y, s1, s2);
-    }
-    __syncthreads();
-    for (int i = tid; i < 2 * kSampWW * kSampWW; i += 256) {
-        const int f = i / (kSampWW * kSampWW), rem = i - f * kSampWW * kSampWW;
-        const int r = rem / kSampWW, c = rem - r * kSampWW;
-        const int y = wy0 + r, x = wx0 + c;
-        const float v = acc[f][r][c];
-        if (v != 0.f && y >= 0 && y < a.H && x >= 0 && x < a.W) atomicAdd((f ? gP2 : gP1) + (int64_t)y * gpitch + x, v);
-    }
+    samples_adjoint_pixel<T>(*a, *gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
+}
+
+// The same with the taps and the gradients of a walk down the columns in
+// registers (k_bw_walk.cuh); four warps per CTA, 32 columns x kBwRows rows
+// each.
+template <typename T, bool GV0>
+__global__ void __launch_bounds__(128, 4) k_bw_samples_walk(const __grid_constant__ IterArgs a,
+                                                            const __grid_constant__ Planes5 gprod, float2 *gV0,
+                                                            float *gP1, float *gP2, int gpitch)
+{
+    bw_samples_walk<T, GV0>(a, gprod, gV0, gP1, gP2, gpitch, [&](int x, int y) {
+        samples_adjoint_general<T>(&a, &gprod, gV0, x, y, gP1, gP2, gpitch);
+    });
 }
 
 // Transpose of the x2 up-sampling: scatter 2 * w * gV0(fine) to the coarse
@@ -498,28 +473,37 @@ cudaError_t box_tile(int kr, Planes5 in, Planes5 out, int H, int W, cudaStream_t
     default: return cudaErrorInvalidValue;
     }
 }
+
+// first: the stage whose V0 is given (its gradient is not wanted).
+template <typename T>
+cudaError_t samples_walk(const IterArgs &a, const Planes5 &A, float2 *gV0, bool first, float *gP1, float *gP2,
+                         int gpitch, cudaStream_t s)
+{
+    const dim3 g((a.W + 31) / 32, (a.H + 4 * kBwRows - 1) / (4 * kBwRows));
+    if (first) k_bw_samples_walk<T, false><<<g, 128, 0, s>>>(a, A, gV0, gP1, gP2, gpitch);
+    else k_bw_samples_walk<T, true><<<g, 128, 0, s>>>(a, A, gV0, gP1, gP2, gpitch);
+    return cudaGetLastError();
+}
 }  // namespace
 
 // One stage of the adjoint.  Window radii 1..10: the solve adjoint from the
 // window sums the forward pass kept (Sk; gS into B, direct part of gV0), the
-// box-sum adjoint tile by tile (gS -> gprod in A), the samples adjoint with
-// the scatter accumulated per tile in shared memory.  Larger radii: one
+// box-sum adjoint tile by tile (gS -> gprod in A), the samples adjoint in a
+// walk down the columns.  Larger radii: one
 // pixel per thread throughout.
 cudaError_t bw_stage(const IterArgs &a, int store, Planes5 Sk, Planes5 A, Planes5 B, const float2 *gV, float2 *gV0,
-                     float *gP1, float *gP2, int gpitch, cudaStream_t s)
+                     bool first, float *gP1, float *gP2, int gpitch, cudaStream_t s)
 {
     const dim3 g = grid2(a.W, a.H), b(32, 8);
     if (block_supports(a.kr)) {
         k_bw_solve<<<g, b, 0, s>>>(Sk, gV, a.vpitch, a.H, a.W, a.eps_rel, a.eps_abs, B, gV0);
         cudaError_t e = box_tile(a.kr, B, A, a.H, a.W, s);
         if (e != cudaSuccess) return e;
-        const dim3 gt((a.W + kSampTS - 1) / kSampTS, (a.H + kSampTS - 1) / kSampTS);
         switch (store) {
-        case ST_F16: k_bw_samples_tile<__half><<<gt, 256, 0, s>>>(a, A, gV0, gP1, gP2, gpitch); break;
-        case ST_BF16: k_bw_samples_tile<__nv_bfloat16><<<gt, 256, 0, s>>>(a, A, gV0, gP1, gP2, gpitch); break;
-        default: k_bw_samples_tile<float><<<gt, 256, 0, s>>>(a, A, gV0, gP1, gP2, gpitch); break;
+        case ST_F16: return samples_walk<__half>(a, A, gV0, first, gP1, gP2, gpitch, s);
+        case ST_BF16: return samples_walk<__nv_bfloat16>(a, A, gV0, first, gP1, gP2, gpitch, s);
+        default: return samples_walk<float>(a, A, gV0, first, gP1, gP2, gpitch, s);
         }
-        return cudaGetLastError();
     }
     switch (store) {
     case ST_F16: k_bw_products<__half><<<g, b, 0, s>>>(a, A); break;
@@ -787,7 +771,7 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
         A.pitch = B.pitch = Sk.pitch = h->pitch[l];
         if (w.Sst[sidx])
             for (int c = 0; c < 5; ++c) Sk.p[c] = w.Sst[sidx] + c * (size_t)h->Hs[l] * h->pitch[l];
-        BW_TRY(bw_stage(a, p.storage, Sk, A, B, gV, gV0, w.gP1[l], w.gP2[l], h->pitch[l], s),
+        BW_TRY(bw_stage(a, p.storage, Sk, A, B, gV, gV0, sidx == 0, w.gP1[l], w.gP2[l], h->pitch[l], s),
                "ofv_backward: stage adjoint");
         if (sidx == 0) break;
         if (t > 0) {

@@ -180,6 +180,39 @@ __device__ __noinline__ void products_general(const T *P1, const T *P2, int H, i
     q[4 * plane] = Gy * r;
 }
 
+// f(lane, bit) for every bit set in the lanes' masks, 32 at a time over the
+// warp (all lanes call).  What the lanes wrote before is visible in f.
+template <typename F>
+__device__ __forceinline__ void warp_compact(unsigned mask, const F &f)
+{
+    if (!__any_sync(0xffffffffu, mask != 0)) return;
+    __syncwarp();
+    const int lane = threadIdx.x & 31, cnt = __popc(mask);
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    for (int base = 0; base < total; base += 32) {
+        const int j = base + lane;
+        int own = 0;  // lanes whose inclusive count is <= j
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const int t = __shfl_sync(0xffffffffu, incl, own + d - 1);
+            if (t <= j) own += d;
+        }
+        unsigned m = __shfl_sync(0xffffffffu, mask, own);
+        int k = j - (__shfl_sync(0xffffffffu, incl, own) - __shfl_sync(0xffffffffu, cnt, own));
+        if (j < total) {
+            for (; k > 0; --k) m &= m - 1;
+            f(own, __ffs(m) - 1);
+        }
+        __syncwarp();
+    }
+}
+
 // Phase 1: the thread walks NROW rows of its column.  Each frame's 4 x 4
 // taps stay in registers and one new row is loaded per step (8 shared loads
 // for a pixel instead of 24), a step ahead at the offset in use; when the
@@ -322,41 +355,15 @@ __device__ __forceinline__ void walk_products(const IterArgs &a, int mode, const
             for (int c = 0; c < 5; ++c) q[c * PLANE + i * P] = p[c];
         }
     }
-    // the warp's pixels for the general sampler, 32 at a time
-    if (__any_sync(0xffffffffu, slow != 0)) {
-        __syncwarp();  // the stand-in products are stored before another lane replaces them
-        const int lane = tid & 31;
-        const int cnt = __popc(slow);
-        int incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += t;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        for (int base = 0; base < total; base += 32) {
-            const int j = base + lane;
-            int own = 0;  // lanes whose inclusive count is <= j
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                const int t = __shfl_sync(0xffffffffu, incl, own + d - 1);
-                if (t <= j) own += d;
-            }
-            unsigned m = __shfl_sync(0xffffffffu, slow, own);
-            int k = j - (__shfl_sync(0xffffffffu, incl, own) - __shfl_sync(0xffffffffu, cnt, own));
-            if (j < total) {
-                for (; k > 0; --k) m &= m - 1;
-                int cx, cr, i0o;
-                WS::item((tid & ~31) + own, cx, cr, i0o);
-                cr += __ffs(m) - 1;
-                const int gx = px0 + cx, gy = py0 + cr;
-                products_general<T, SP>(static_cast<const T *>(a.P1), static_cast<const T *>(a.P2), H, W, a.pitch,
-                                        st1, st2, sx0, sy0, gx, gy, fetch_v0_rt<COH>(a, mode, gx, gy),
-                                        prod + cr * P + cx, PLANE);
-            }
-            __syncwarp();
-        }
-    }
+    // the warp's pixels for the general sampler
+    warp_compact(slow, [&](int own, int row) {
+        int cx, cr, i0o;
+        WS::item((tid & ~31) + own, cx, cr, i0o);
+        cr += row;
+        const int gx = px0 + cx, gy = py0 + cr;
+        products_general<T, SP>(static_cast<const T *>(a.P1), static_cast<const T *>(a.P2), H, W, a.pitch, st1, st2, sx0,
+                                sy0, gx, gy, fetch_v0_rt<COH>(a, mode, gx, gy), prod + cr * P + cx, PLANE);
+    });
 }
 
 __device__ __forceinline__ float add_v(float a, float b) { return a + b; }
