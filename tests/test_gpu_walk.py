@@ -70,7 +70,7 @@ def test_fields_at_unaligned_addresses():
         assert np.array_equal(v.cpu().numpy().reshape(H, W), a[1])
 
 
-@pytest.mark.parametrize("H,W,kr,shift", [(31, 33, 4, (0.8, -0.5)), (32, 64, 2, (0.8, -0.5)), (65, 31, 8, (-1.2, 0.4)),
+@pytest.mark.parametrize("H,W,kr,shift", [(31, 33, 4, (0.8, -0.5)), (32, 64, 3, (0.8, -0.5)), (65, 31, 8, (-1.2, 0.4)),
                                           (40, 56, 10, (0.3, 0.2)), (96, 80, 4, (9.3, -8.7))])
 def test_samples_adjoint_at_remainders_matches_oracle(H, W, kr, shift):
     psl = 2 if abs(shift[0]) > 4 else 0
