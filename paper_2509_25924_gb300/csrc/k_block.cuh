@@ -44,6 +44,7 @@ struct BlockParams {
     int mode;                    // V0Mode, uniform per launch
     int use_tma;                 // 1: tm[k] maps the two level images of pair k
     int *err;                    // error word (set to 1 when a TMA wait expires), or null
+    int overlap;                 // see launch_iter_block
     int row0, row1;              // output rows of the launch (row0 a multiple of the radius's tile edge)
     CUtensorMap tm[kBlockMaxBatch][2];
 };
@@ -865,13 +866,16 @@ struct QueueParams {
 
 // Host launchers, explicitly instantiated per level storage type T and kind
 // of iteration in k_block_{f32,f16,bf16}.cu (ITER_BOX) and
-// k_block_var_{f32,f16,bf16}.cu (ITER_KEEP and ITER_VAR).
+// k_block_var_{f32,f16,bf16}.cu (ITER_KEEP and ITER_VAR) and
+// k_block_chain_{f32,f16,bf16}.cu (ITER_CHAIN).
 // shape: the tile shape v (ITER_KEEP and ITER_VAR have the default shape
-// only; the batched launch has no ITER_KEEP)
+// only; the batched launch has ITER_BOX and ITER_VAR)
 enum IterKind : int {
     ITER_BOX = 0,   // uniform box window (k_walk.cuh)
     ITER_KEEP = 1,  // the same, keeping the window sums for the reverse mode
-    ITER_VAR = 2    // estimator variants: Gaussian window, increment form, region mask
+    ITER_VAR = 2,   // estimator variants: Gaussian window, increment form, region mask
+    ITER_CHAIN = 3  // ITER_BOX in a chain of launches that overlap their ends (a kernel of its own: the
+                    // two instructions cost a stream of plain launches 2 %)
 };
 template <typename T, int KIND>
 cudaError_t launch_block_t(const BlockParams &p, int kr, int npairs, cudaStream_t s, int shape = 0);

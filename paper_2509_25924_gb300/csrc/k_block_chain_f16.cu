@@ -1,0 +1,9 @@
+// Iteration kernels for __half level storage, window radii 1..10, for a chain
+// of launches on one stream (one pair).
+#include "k_block_inst.cuh"
+
+namespace ofv {
+
+OFV_INSTANTIATE_BLOCK(__half, ITER_CHAIN)
+
+}  // namespace ofv

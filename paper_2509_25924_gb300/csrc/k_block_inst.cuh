@@ -42,8 +42,9 @@ __global__ void __launch_bounds__(IterShape<T, KS, KIND>::NT, IterShape<T, KS, K
         block_tile<T, KS, false>(prm.a[z], prm.mode, blockIdx.x, prm.row0 / IterShape<T, KS, KIND>::TY + blockIdx.y, smem_f4,
                                  tm1, tm2, prm.err, s_bar);
     } else {
-        walk_tile<T, typename IterShape<T, KS, KIND>::WS, false, KIND == ITER_KEEP>(
-            prm.a[z], prm.mode, blockIdx.x, blockIdx.y, prm.row0, prm.row1, smem_f4, tm1, tm2, prm.err, s_bar);
+        walk_tile<T, typename IterShape<T, KS, KIND>::WS, false, KIND == ITER_KEEP, KIND == ITER_CHAIN>(
+            prm.a[z], prm.mode, blockIdx.x, blockIdx.y, prm.row0, prm.row1, smem_f4, tm1, tm2, prm.err, s_bar,
+            prm.overlap == 2);
     }
 }
 
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(IterShape<T, KS, KIND>::NT, IterShape<T, KS, K
     if constexpr (VAR) {
         block_tile<T, KS, true>(o.a, o.mode, o.bx, o.by, smem_f4, tm1, tm2, q.tma_err, s_bar);
     } else {
-        walk_tile<T, typename IterShape<T, KS, KIND>::WS, true, false>(o.a, o.mode, o.bx, o.by, 0, o.a.H, smem_f4, tm1,
-                                                                       tm2, q.tma_err, s_bar);
+        walk_tile<T, typename IterShape<T, KS, KIND>::WS, true, false, false>(o.a, o.mode, o.bx, o.by, 0, o.a.H, smem_f4, tm1,
+                                                                       tm2, q.tma_err, s_bar, false);
     }
     __threadfence();
     __syncthreads();
@@ -166,8 +167,7 @@ cudaError_t run_block(const BlockParams &p, dim3 grid, int dev, cudaStream_t s)
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) granted[dev] = smem;
     }
-    kern<<<grid, IterShape<T, KS, KIND>::NT, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_after(KIND == ITER_CHAIN, kern, grid, dim3(IterShape<T, KS, KIND>::NT), smem, s, p);
 }
 
 // KS = kr + 16 shape for the radii and shapes instantiated here: every
@@ -176,7 +176,7 @@ cudaError_t run_block(const BlockParams &p, dim3 grid, int dev, cudaStream_t s)
 template <int KIND>
 constexpr int ks_of(int kr, int shape)
 {
-    return (kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1 || (KIND != ITER_BOX && shape != 0)) ? 0 : kr + 16 * shape;
+    return (kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1 || (KIND != ITER_BOX && KIND != ITER_CHAIN && shape != 0)) ? 0 : kr + 16 * shape;
 }
 
 #define OFV_KS_CASES(X)                                                                                    \
@@ -194,7 +194,7 @@ cudaError_t launch_block_t(const BlockParams &p, int kr, int npairs, cudaStream_
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX) { X##_BODY(K) } else { break; }
+        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
 #define OFV_BLOCK_CASE(K) case K: OFV_BLOCK_CASE_BODY(K)
 #define OFV_BLOCK_CASE_BODY(K)                                                                             \
     {                                                                                                      \
@@ -252,7 +252,7 @@ cudaError_t launch_queue_t(const QueueParams &q, int kr, cudaStream_t s, int sha
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX) { X##_BODY(K) } else { break; }
+        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
 #define OFV_QUEUE_CASE(K) case K: OFV_QUEUE_CASE_BODY(K)
 #define OFV_QUEUE_CASE_BODY(K) return run_queue<T, QKS(K), KIND>(q, dev, s);
     OFV_KS_CASES(OFV_QUEUE_CASE)
@@ -271,7 +271,7 @@ int queue_occupancy_t(int kr, int shape)
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX) { X##_BODY(K) } else { break; }
+        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
 #define OFV_OCC_CASE(K) case K: OFV_OCC_CASE_BODY(K)
 #define OFV_OCC_CASE_BODY(K) return queue_occupancy_kr<T, QKS(K), KIND>();
     OFV_KS_CASES(OFV_OCC_CASE)

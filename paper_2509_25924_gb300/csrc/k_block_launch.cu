@@ -7,6 +7,9 @@
 namespace ofv {
 
 extern template cudaError_t launch_block_t<float, ITER_BOX>(const BlockParams &, int, int, cudaStream_t, int);
+extern template cudaError_t launch_block_t<float, ITER_CHAIN>(const BlockParams &, int, int, cudaStream_t, int);
+extern template cudaError_t launch_block_t<__half, ITER_CHAIN>(const BlockParams &, int, int, cudaStream_t, int);
+extern template cudaError_t launch_block_t<__nv_bfloat16, ITER_CHAIN>(const BlockParams &, int, int, cudaStream_t, int);
 extern template cudaError_t launch_block_t<float, ITER_KEEP>(const BlockParams &, int, int, cudaStream_t, int);
 extern template cudaError_t launch_block_t<float, ITER_VAR>(const BlockParams &, int, int, cudaStream_t, int);
 extern template cudaError_t launch_block_t<__half, ITER_BOX>(const BlockParams &, int, int, cudaStream_t, int);
@@ -55,6 +58,7 @@ cudaError_t launch_kind(const BlockParams &p, int kind, int kr, int npairs, cuda
 {
     switch (kind) {
     case ITER_VAR: return launch_block_t<T, ITER_VAR>(p, kr, npairs, s, shape);
+    case ITER_CHAIN: return launch_block_t<T, ITER_CHAIN>(p, kr, npairs, s, shape);
     case ITER_KEEP: return launch_block_t<T, ITER_KEEP>(p, kr, npairs, s, shape);
     default: return launch_block_t<T, ITER_BOX>(p, kr, npairs, s, shape);
     }
@@ -62,7 +66,7 @@ cudaError_t launch_kind(const BlockParams &p, int kind, int kr, int npairs, cuda
 }  // namespace
 
 cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode, cudaStream_t s,
-                              const CUtensorMap *const *tm, int *err, int row0, int nrows, int shape)
+                              const CUtensorMap *const *tm, int *err, int row0, int nrows, int shape, int overlap)
 {
     if (npairs < 1 || npairs > kBlockMaxBatch || !block_supports(a[0].kr)) return cudaErrorInvalidValue;
     BlockParams p;
@@ -71,6 +75,7 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
     p.mode = mode;
     p.err = err;
     p.row0 = row0;
+    p.overlap = overlap;
     p.row1 = nrows > 0 ? row0 + nrows : a[0].H;
     p.use_tma = 0;
     if (tm) {
@@ -86,8 +91,9 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
     }
     // the kernels with variant code only when a variant is on, and those that
     // keep the window sums only for the reverse mode (uniform per launch)
-    const int kind = a[0].inc || a[0].gauss || a[0].mask ? ITER_VAR : a[0].s_out ? ITER_KEEP : ITER_BOX;
-    if (kind != ITER_BOX && shape != 0) {
+    const bool var = a[0].inc || a[0].gauss || a[0].mask;
+    const int kind = var ? ITER_VAR : a[0].s_out ? ITER_KEEP : overlap ? ITER_CHAIN : ITER_BOX;
+    if ((kind == ITER_VAR || kind == ITER_KEEP) && shape != 0) {
         // these have the default tile shape only; tensor maps made for
         // another shape's box would not match theirs
         p.use_tma = 0;
@@ -100,7 +106,7 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
         block_stage_box(store, a[0].kr, &c1, &r1, 0, true);
         if (c0 != c1 || r0 != r1) p.use_tma = 0;
     }
-    if (kind == ITER_BOX && shape == 0 && npairs == 1 && walk_small_tiles(a[0].kr, a[0].W, p.row1 - row0)) shape = 1;
+    if ((kind == ITER_BOX || kind == ITER_CHAIN) && shape == 0 && npairs == 1 && walk_small_tiles(a[0].kr, a[0].W, p.row1 - row0)) shape = 1;
     switch (store) {
     case ST_F16: return launch_kind<__half>(p, kind, a[0].kr, npairs, s, shape);
     case ST_BF16: return launch_kind<__nv_bfloat16>(p, kind, a[0].kr, npairs, s, shape);

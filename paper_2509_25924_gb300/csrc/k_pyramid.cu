@@ -38,6 +38,7 @@ struct IngestList {
 template <typename TI, typename TS, typename FR>
 __global__ void __launch_bounds__(256) k_ingest(const __grid_constant__ FR p)
 {
+    pdl_trigger();
     const IngestArgs &a = p.get(blockIdx.z);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(256) k_ingest(const __grid_constant__ FR p)
 template <int NRC, typename TI, typename TS, typename FR>
 __device__ __forceinline__ void ingest_norm_tile(const FR &p)
 {
+    pdl_trigger();
     extern __shared__ float tile[];  // (32 + 2 NR) rows of (32 + 2 NR), then (32 + 2 NR) x 32 row sums
     const IngestArgs &a = p.get(blockIdx.z);
     const int nr = NRC > 0 ? NRC : a.nr, K = 2 * nr + 1;
@@ -213,6 +215,7 @@ __device__ __forceinline__ void store8(__nv_bfloat16 *d, const float f[8])
 template <typename TI, typename TS, typename FR>
 __global__ void __launch_bounds__(256) k_ingest8(const __grid_constant__ FR p)
 {
+    pdl_trigger();
     const IngestArgs &a = p.get(blockIdx.z);
     const int W8 = a.W >> 3;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -235,6 +238,8 @@ __global__ void __launch_bounds__(256) k_ingest8(const __grid_constant__ FR p)
 template <typename TS, typename FR>
 __global__ void __launch_bounds__(256) k_prefilter(const __grid_constant__ FR p)
 {
+    pdl_wait();
+    pdl_trigger();
     const IngestArgs &a = p.get(blockIdx.z);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
@@ -253,7 +258,7 @@ __global__ void __launch_bounds__(256) k_prefilter(const __grid_constant__ FR p)
 // the grid, which covers the largest frame); p: the same frames as the
 // kernels read them.
 template <typename TS, typename FR>
-static cudaError_t ingest_t(const FR &p, const IngestArgs *f, int nframes, cudaStream_t s)
+static cudaError_t ingest_t(const FR &p, const IngestArgs *f, int nframes, cudaStream_t s, bool overlap = false)
 {
     const IngestArgs &a = f[0];
     bool vec = a.nr == 0 && !a.prefilter;
@@ -291,22 +296,23 @@ static cudaError_t ingest_t(const FR &p, const IngestArgs *f, int nframes, cudaS
         default: k_ingest<float, TS, FR><<<grd, blk, 0, s>>>(p); break;
         }
     }
-    if (a.prefilter) k_prefilter<TS, FR><<<grd, blk, 0, s>>>(p);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && a.prefilter) e = launch_after(overlap, k_prefilter<TS, FR>, grd, blk, 0, s, p);
+    return e;
 }
 
 // Ingest nframes (1 .. kMaxFramesPerLaunch) frames in one launch
 // (gridDim.z = nframes).
-cudaError_t launch_ingest_frames(const IngestArgs *f, int nframes, int store, cudaStream_t s)
+cudaError_t launch_ingest_frames(const IngestArgs *f, int nframes, int store, cudaStream_t s, bool overlap)
 {
     if (nframes < 1 || nframes > kMaxFramesPerLaunch) return cudaErrorInvalidValue;
     IngestPair p;
     for (int k = 0; k < nframes; ++k) p.f[k] = f[k];
     p.scale = f[0].in_type == IN_F32 ? 1.0f : 1.0f / (float)((1u << f[0].bits) - 1u);
     switch (store) {
-    case ST_F16: return ingest_t<__half>(p, f, nframes, s);
-    case ST_BF16: return ingest_t<__nv_bfloat16>(p, f, nframes, s);
-    default: return ingest_t<float>(p, f, nframes, s);
+    case ST_F16: return ingest_t<__half>(p, f, nframes, s, overlap);
+    case ST_BF16: return ingest_t<__nv_bfloat16>(p, f, nframes, s, overlap);
+    default: return ingest_t<float>(p, f, nframes, s, overlap);
     }
 }
 
@@ -364,6 +370,8 @@ __device__ __forceinline__ void load7<float>(const float *row, int c0, int Ws, b
 template <typename TS, typename FR>
 __global__ void __launch_bounds__(256) k_reduce(const __grid_constant__ FR p)
 {
+    pdl_wait();
+    pdl_trigger();
     const ReduceArgs &a = p.get(blockIdx.z);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
@@ -395,7 +403,7 @@ __global__ void __launch_bounds__(256) k_reduce(const __grid_constant__ FR p)
 
 // The grid covers the largest output of the frames (each exits outside its own).
 template <typename FR>
-static cudaError_t reduce_t(const FR &p, const ReduceArgs *f, int nframes, int store, cudaStream_t s)
+static cudaError_t reduce_t(const FR &p, const ReduceArgs *f, int nframes, int store, cudaStream_t s, bool overlap = false)
 {
     int Hd = 0, Wd = 0;
     for (int k = 0; k < nframes; ++k) {
@@ -405,20 +413,19 @@ static cudaError_t reduce_t(const FR &p, const ReduceArgs *f, int nframes, int s
     dim3 blk(32, 8);
     dim3 grd(((Wd + 1) / 2 + 31) / 32, (Hd + 7) / 8, nframes);
     switch (store) {
-    case ST_F16: k_reduce<__half, FR><<<grd, blk, 0, s>>>(p); break;
-    case ST_BF16: k_reduce<__nv_bfloat16, FR><<<grd, blk, 0, s>>>(p); break;
-    default: k_reduce<float, FR><<<grd, blk, 0, s>>>(p); break;
+    case ST_F16: return launch_after(overlap, k_reduce<__half, FR>, grd, blk, 0, s, p);
+    case ST_BF16: return launch_after(overlap, k_reduce<__nv_bfloat16, FR>, grd, blk, 0, s, p);
+    default: return launch_after(overlap, k_reduce<float, FR>, grd, blk, 0, s, p);
     }
-    return cudaGetLastError();
 }
 
 // Reduce one level of nframes (1 .. kMaxFramesPerLaunch) frames in one launch.
-cudaError_t launch_reduce_frames(const ReduceArgs *f, int nframes, int store, cudaStream_t s)
+cudaError_t launch_reduce_frames(const ReduceArgs *f, int nframes, int store, cudaStream_t s, bool overlap)
 {
     if (nframes < 1 || nframes > kMaxFramesPerLaunch) return cudaErrorInvalidValue;
     ReducePair p;
     for (int k = 0; k < nframes; ++k) p.f[k] = f[k];
-    return reduce_t(p, f, nframes, store, s);
+    return reduce_t(p, f, nframes, store, s, overlap);
 }
 
 // Any number of frames (of any sizes) in one launch (see launch_ingest_list).

@@ -524,10 +524,12 @@ __device__ __forceinline__ void walk_fill_border(T *stage, int sx0, int sy0, int
 // One tile (the CTA's only one): the output pixels from (bx TX, row0 + by TY)
 // on, rows below row1 and the level's end.  TMA staging needs tensor maps
 // tm1, tm2 (box SP x SHB), or null, and NBAND mbarriers in shared memory.
-template <typename T, typename WS, bool COH, bool KEEP>
+// CHAIN: the launch may have started before the one ahead of it ended; its
+// images are staged ahead of the wait for that launch if early.
+template <typename T, typename WS, bool COH, bool KEEP, bool CHAIN>
 __device__ __forceinline__ void walk_tile(const IterArgs &a, int mode, int bx, int by, int row0, int row1,
                                           float4 *smem_f4, const CUtensorMap *tm1, const CUtensorMap *tm2, int *err,
-                                          uint64_t *tma_bars)
+                                          uint64_t *tma_bars, bool early)
 {
     using SS = WalkStage<T, WS>;
     constexpr int TX = WS::TX, TY = WS::TY, R = WS::R, RW = WS::RW, P = WS::P, PLANE = WS::PLANE, NT = WS::NT;
@@ -545,6 +547,7 @@ __device__ __forceinline__ void walk_tile(const IterArgs &a, int mode, int bx, i
     uint64_t *bars = nullptr;
 
     // phase 0
+    if (CHAIN && !early) pdl_wait();
     if (tm1 != nullptr) {
         if (tid == 0) {
             mbar_init_n<NBAND>(tma_bars);
@@ -584,6 +587,11 @@ __device__ __forceinline__ void walk_tile(const IterArgs &a, int mode, int bx, i
     if (!interior) {
         walk_fill_border<T, WS>(stage, sx0, sy0, H, W);
         __syncthreads();
+    }
+
+    if (CHAIN) {
+        if (early) pdl_wait();
+        pdl_trigger();
     }
 
     // phase 1

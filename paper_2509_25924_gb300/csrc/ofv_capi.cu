@@ -188,7 +188,7 @@ void encode_tensor_maps(ofv_handle *h)
 // Steps 1-2: ingest nf frames (frames[k] into pyramid slot slots[k]) and
 // reduce them, nf frames per launch.
 ofv_status build_pyramids(ofv_handle *h, const void *const *frames, const int *slots, int nf, cudaStream_t s,
-                          int tset = 0)
+                          int tset = 0, bool overlap = false)
 {
     const ofv_params &p = h->p;
     const int sb = store_bytes(p.storage), ib = input_bytes(p.input);
@@ -215,7 +215,7 @@ ofv_status build_pyramids(ofv_handle *h, const void *const *frames, const int *s
     {
         const double N = (double)h->H * h->W;
         ProfScope ps(h, s, OFV_K_INGEST, nf * N * (ib + sb));
-        ofv_status st = last_launch(launch_ingest_frames(ia, nf, p.storage, s), "ingest launch");
+        ofv_status st = last_launch(launch_ingest_frames(ia, nf, p.storage, s, overlap), "ingest launch");
         if (st != OFV_OK) return st;
     }
     for (int l = 1; l < h->L; ++l) {
@@ -233,7 +233,7 @@ ofv_status build_pyramids(ofv_handle *h, const void *const *frames, const int *s
         }
         const double bytes = nf * (double)sb * ((double)h->Hs[l - 1] * h->Ws[l - 1] + (double)h->Hs[l] * h->Ws[l]);
         ProfScope ps(h, s, OFV_K_REDUCE, bytes);
-        ofv_status st = last_launch(launch_reduce_frames(ra, nf, p.storage, s), "reduce launch");
+        ofv_status st = last_launch(launch_reduce_frames(ra, nf, p.storage, s, overlap), "reduce launch");
         if (st != OFV_OK) return st;
     }
     return OFV_OK;
@@ -244,7 +244,8 @@ ofv_status build_pyramids(ofv_handle *h, const void *const *frames, const int *s
 // start) pair k starts its coarsest level from the level-0 field iu[k],
 // iv[k] (H x W dense) decimated to that level, else from zero.
 ofv_status run_levels(ofv_handle *h, int np, const int *s1, const int *s2, float *const *u, float *const *v,
-                      cudaStream_t s, int vset = 0, const float *const *iu = nullptr, const float *const *iv = nullptr)
+                      cudaStream_t s, int vset = 0, const float *const *iu = nullptr, const float *const *iv = nullptr,
+                     bool overlap = false)
 {
     const ofv_params &p = h->p;
     const int sb = store_bytes(p.storage);
@@ -328,8 +329,9 @@ ofv_status run_levels(ofv_handle *h, int np, const int *s1, const int *s2, float
                     tm[2 * k + 1] = &h->tmap[s2[k]][l];
                 }
                 const bool use = h->tma_ok[l] && h->tma_err_d;
+                const bool first = l == h->L - 1 && t == 0;  // after the pyramid's launches
                 e = launch_iter_block(a, np, p.storage, mode, s, use ? tm : nullptr, h->tma_err_d, 0, 0,
-                                      tile_shape_of(p));
+                                      tile_shape_of(p), !overlap ? 0 : first ? 1 : 2);
             } else {
                 for (int k = 0; k < np && e == cudaSuccess; ++k)
                     e = p.path == OFV_PATH_PLAIN ? launch_iter_plain(a[k], h->plain, p.storage, mode, s)
@@ -810,13 +812,18 @@ ofv_status ofv_compute(ofv_handle *h, const void *I1, const void *I2, float *u, 
     cudaStream_t cs = (cudaStream_t)s;
     const void *fr[2] = {I1, I2};
     const int slots[2] = {0, 1};
-    st = build_pyramids(h, fr, slots, 2, cs);
+    // One pair's launches follow one another on one stream: each may start
+    // while the last wave of the one ahead of it drains, and its tiles stage
+    // their images meanwhile.  (The groups of a sequence run on several
+    // streams, whose launches fill each other's ends.)
+    const bool overlap = !h->prof;
+    st = build_pyramids(h, fr, slots, 2, cs, 0, overlap);
     if (st != OFV_OK) return st;
     h->last_s1 = 0;
     h->last_s2 = 1;
     const int s1[1] = {0}, s2[1] = {1};
     float *uu[1] = {u}, *vv[1] = {v};
-    return run_levels(h, 1, s1, s2, uu, vv, cs);
+    return run_levels(h, 1, s1, s2, uu, vv, cs, 0, nullptr, nullptr, overlap);
 }
 
 ofv_status ofv_compute_host(ofv_handle *h, const void *I1, const void *I2, float *u, float *v, ofv_stream_t s)

@@ -26,6 +26,39 @@ constexpr int kMaxPairsPerLaunch = 8;
 constexpr int kMaxWindowRadius = 16;  // largest KR
 constexpr int kMaxFramesPerLaunch = kMaxPairsPerLaunch + 1;
 
+// Programmatic dependent launch: a kernel launched by launch_after may start
+// while the kernel before it on the stream still runs, from the moment every
+// CTA of that kernel has called pdl_trigger; pdl_wait returns when it has
+// completed and its writes are visible.  Every kernel launched so waits before
+// it reads or writes what earlier work on the stream touches, and triggers
+// only after its own wait -- so whatever precedes the kernel before it is
+// complete even ahead of the wait.  Both are no-ops after a plain launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Args>
+inline cudaError_t launch_after(bool overlap, void (*kern)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                const Args &...args)
+{
+    if (!overlap) {
+        kern<<<grid, block, smem, s>>>(args...);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here
+    return e;
+}
+
 // Level images are stored with a row pitch (elements) that is a multiple of
 // 64, so every row starts 128-byte aligned in all storage types.
 constexpr int kPitchAlign = 64;
@@ -89,11 +122,14 @@ bool block_supports(int kr);
 cudaError_t launch_recip(const float *x, float *y, int n, cudaStream_t s);
 // row0, nrows: output rows row0 .. row0+nrows-1 only, row0 a multiple of the
 // tile edge (nrows 0: to the bottom of the level).
+// overlap: 0 a plain launch; 1 may start before the launch ahead of it on the
+// stream has ended (launch_after); 2 that launch is an iteration too, so the
+// level images are complete and staging starts ahead of the wait.
 // shape: the tile shape (0 default, 1 the alternative; the estimator
 // variants run the default shape).
 cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode, cudaStream_t s,
                               const CUtensorMap *const *tm = nullptr, int *err = nullptr, int row0 = 0, int nrows = 0,
-                              int shape = 0);
+                              int shape = 0, int overlap = 0);
 // TMA box of the iteration kernels' staging (columns, rows of one band) for
 // this storage, radius and tile shape; var: of the estimator variants'
 // kernels (Gaussian window, increment form).
@@ -120,14 +156,15 @@ struct IngestArgs {
     int prefilter;
 };
 // Ingest nframes (1 or 2) frames in one launch.
-cudaError_t launch_ingest_frames(const IngestArgs *f, int nframes, int store, cudaStream_t s);
+// Kernels after the first start ahead (launch_after) with overlap.
+cudaError_t launch_ingest_frames(const IngestArgs *f, int nframes, int store, cudaStream_t s, bool overlap = false);
 
 struct ReduceArgs {
     const void *src; int Hs, Ws, spitch;
     void *dst; int Hd, Wd, dpitch;
 };
 // Reduce one level of nframes (1 or 2) frames in one launch.
-cudaError_t launch_reduce_frames(const ReduceArgs *f, int nframes, int store, cudaStream_t s);
+cudaError_t launch_reduce_frames(const ReduceArgs *f, int nframes, int store, cudaStream_t s, bool overlap = false);
 
 // Any number of frames of any sizes in one launch: f on the host, dev_f the
 // same descriptors in device memory, valid until the launch has run.
