@@ -81,6 +81,8 @@ __global__ void k_bw_box(Planes5 in, Planes5 out, int H, int W, int kr, int dir)
 __global__ void k_bw_solve(Planes5 S, const float2 *gV, int vpitch, int H, int W, float eps_rel, float eps_abs,
                            Planes5 gS, float2 *gV0)
 {
+    pdl_wait();
+    pdl_trigger();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= W || y >= H) return;
@@ -180,12 +182,12 @@ __device__ __forceinline__ void sample_adj(const T *P, int H, int W, int pitch, 
 // warped samples at pixel (x, y); adds into gV0 and, through add1 and add2,
 // into the level-image gradients.
 template <typename T, typename Scatter>
-__device__ __forceinline__ void samples_adjoint_pixel(const IterArgs &a, const Planes5 &gprod, float2 *gV0, int x,
-                                                      int y, const Scatter &add1, const Scatter &add2)
+__device__ __forceinline__ void samples_adjoint_pixel(const IterArgs &a, int mode, const Planes5 &gprod, float2 *gV0,
+                                                      int x, int y, const Scatter &add1, const Scatter &add2)
 {
     const T *P1 = static_cast<const T *>(a.P1);
     const T *P2 = static_cast<const T *>(a.P2);
-    const float2 V0 = fetch_v0<V0_SAME>(a, x, y);
+    const float2 V0 = fetch_v0_rt<false>(a, mode, x, y);
     const float hx = 0.5f * V0.x, hy = 0.5f * V0.y;
     const Sample s1 = sample_level(P1, a.H, a.W, a.pitch, x, y, -hx, -hy);
     const Sample s2 = sample_level(P2, a.H, a.W, a.pitch, x, y, hx, hy);
@@ -214,28 +216,30 @@ __global__ void k_bw_samples(IterArgs a, Planes5 gprod, float2 *gV0, float *gP1,
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= a.W || y >= a.H) return;
-    samples_adjoint_pixel<T>(a, gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
+    samples_adjoint_pixel<T>(a, V0_SAME, gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
 }
 
 // The walk's pixels that need the general form: a call, which keeps the
 // walk's registers apart from it.
 template <typename T>
-__device__ __noinline__ void samples_adjoint_general(const IterArgs *a, const Planes5 *gprod, float2 *gV0, int x, int y,
-                                                     float *gP1, float *gP2, int gpitch)
+__device__ __noinline__ void samples_adjoint_general(const IterArgs *a, int mode, const Planes5 *gprod, float2 *gV0,
+                                                     int x, int y, float *gP1, float *gP2, int gpitch)
 {
-    samples_adjoint_pixel<T>(*a, *gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
+    samples_adjoint_pixel<T>(*a, mode, *gprod, gV0, x, y, ScatterGlobal{gP1, gpitch}, ScatterGlobal{gP2, gpitch});
 }
 
 // The same with the taps and the gradients of a walk down the columns in
 // registers (k_bw_walk.cuh); four warps per CTA, 32 columns x kBwRows rows
 // each.
 template <typename T, bool GV0>
-__global__ void __launch_bounds__(128, 4) k_bw_samples_walk(const __grid_constant__ IterArgs a,
+__global__ void __launch_bounds__(128, 4) k_bw_samples_walk(const __grid_constant__ IterArgs a, int mode,
                                                             const __grid_constant__ Planes5 gprod, float2 *gV0,
                                                             float *gP1, float *gP2, int gpitch)
 {
-    bw_samples_walk<T, GV0>(a, gprod, gV0, gP1, gP2, gpitch, [&](int x, int y) {
-        samples_adjoint_general<T>(&a, &gprod, gV0, x, y, gP1, gP2, gpitch);
+    pdl_wait();
+    pdl_trigger();
+    bw_samples_walk<T, GV0>(a, mode, gprod, gV0, gP1, gP2, gpitch, [&](int x, int y) {
+        samples_adjoint_general<T>(&a, mode, &gprod, gV0, x, y, gP1, gP2, gpitch);
     });
 }
 
@@ -476,13 +480,12 @@ cudaError_t box_tile(int kr, Planes5 in, Planes5 out, int H, int W, cudaStream_t
 
 // first: the stage whose V0 is given (its gradient is not wanted).
 template <typename T>
-cudaError_t samples_walk(const IterArgs &a, const Planes5 &A, float2 *gV0, bool first, float *gP1, float *gP2,
+cudaError_t samples_walk(const IterArgs &a, int mode, const Planes5 &A, float2 *gV0, bool first, float *gP1, float *gP2,
                          int gpitch, cudaStream_t s)
 {
     const dim3 g((a.W + 31) / 32, (a.H + 4 * kBwRows - 1) / (4 * kBwRows));
-    if (first) k_bw_samples_walk<T, false><<<g, 128, 0, s>>>(a, A, gV0, gP1, gP2, gpitch);
-    else k_bw_samples_walk<T, true><<<g, 128, 0, s>>>(a, A, gV0, gP1, gP2, gpitch);
-    return cudaGetLastError();
+    return launch_after(true, first ? k_bw_samples_walk<T, false> : k_bw_samples_walk<T, true>, g, dim3(128), 0, s, a, mode,
+                        A, gV0, gP1, gP2, gpitch);
 }
 }  // namespace
 
@@ -491,18 +494,19 @@ cudaError_t samples_walk(const IterArgs &a, const Planes5 &A, float2 *gV0, bool 
 // box-sum adjoint tile by tile (gS -> gprod in A), the samples adjoint in a
 // walk down the columns.  Larger radii: one
 // pixel per thread throughout.
-cudaError_t bw_stage(const IterArgs &a, int store, Planes5 Sk, Planes5 A, Planes5 B, const float2 *gV, float2 *gV0,
+cudaError_t bw_stage(const IterArgs &a, int mode, int store, Planes5 Sk, Planes5 A, Planes5 B, const float2 *gV, float2 *gV0,
                      bool first, float *gP1, float *gP2, int gpitch, cudaStream_t s)
 {
     const dim3 g = grid2(a.W, a.H), b(32, 8);
     if (block_supports(a.kr)) {
-        k_bw_solve<<<g, b, 0, s>>>(Sk, gV, a.vpitch, a.H, a.W, a.eps_rel, a.eps_abs, B, gV0);
-        cudaError_t e = box_tile(a.kr, B, A, a.H, a.W, s);
+        cudaError_t e = launch_after(true, k_bw_solve, g, b, 0, s, Sk, gV, a.vpitch, a.H, a.W, a.eps_rel, a.eps_abs, B,
+                                     gV0);
+        if (e == cudaSuccess) e = box_tile(a.kr, B, A, a.H, a.W, s);
         if (e != cudaSuccess) return e;
         switch (store) {
-        case ST_F16: return samples_walk<__half>(a, A, gV0, first, gP1, gP2, gpitch, s);
-        case ST_BF16: return samples_walk<__nv_bfloat16>(a, A, gV0, first, gP1, gP2, gpitch, s);
-        default: return samples_walk<float>(a, A, gV0, first, gP1, gP2, gpitch, s);
+        case ST_F16: return samples_walk<__half>(a, mode, A, gV0, first, gP1, gP2, gpitch, s);
+        case ST_BF16: return samples_walk<__nv_bfloat16>(a, mode, A, gV0, first, gP1, gP2, gpitch, s);
+        default: return samples_walk<float>(a, mode, A, gV0, first, gP1, gP2, gpitch, s);
         }
     }
     switch (store) {
@@ -641,7 +645,9 @@ size_t bw_layout(const ofv_handle *h, char *base, BwLayout *o)
                         : nullptr;
     }
     for (int l = 0; l < L; ++l)
-        o->V0in[l] = reinterpret_cast<float2 *>(take((size_t)h->Hs[l] * h->pitch[l] * sizeof(float2)));
+        o->V0in[l] = block_supports(h->p.kernel_radius)
+                         ? nullptr
+                         : reinterpret_cast<float2 *>(take((size_t)h->Hs[l] * h->pitch[l] * sizeof(float2)));
     const size_t plane = (size_t)h->Hs[0] * h->pitch[0];
     for (int c = 0; c < 5; ++c) {
         o->A.p[c] = reinterpret_cast<float *>(take(plane * sizeof(float)));
@@ -715,6 +721,7 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
     h->last_s1 = 0;
     h->last_s2 = 1;
     const int L = h->L, IT = p.iterations, S = L * IT;
+    const bool block = block_supports(p.kernel_radius);
     auto stage_args = [&](int sidx) {
         const int l = L - 1 - sidx / IT, t = sidx % IT;
         IterArgs a;
@@ -728,13 +735,26 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
         a.kr = p.kernel_radius;
         a.eps_rel = p.det_rel_eps;
         a.eps_abs = p.det_abs_eps;
-        a.V0 = t == 0 ? w.V0in[l] : w.Vst[sidx - 1];
+        // V0 of a level's first stage: radii up to 10 read it where it is
+        // (zero, or up-sampled from the coarser level's last field), larger
+        // ones from a plane
+        if (t > 0) {
+            a.V0 = w.Vst[sidx - 1];
+        } else if (!block) {
+            a.V0 = w.V0in[l];
+        } else if (sidx > 0) {
+            a.Vc = w.Vst[sidx - 1];
+            a.Hc = h->Hs[l + 1];
+            a.Wc = h->Ws[l + 1];
+            a.vcpitch = h->pitch[l + 1];
+        }
         return a;
     };
+    auto stage_mode = [&](int sidx) { return !block || sidx % IT > 0 ? V0_SAME : sidx == 0 ? V0_ZERO : V0_UP; };
     for (int sidx = 0; sidx < S; ++sidx) {
         const int l = L - 1 - sidx / IT, t = sidx % IT;
         IterArgs a = stage_args(sidx);
-        if (t == 0) {
+        if (t == 0 && !block) {
             IterArgs b = a;
             int mode = V0_ZERO;
             if (sidx > 0) {
@@ -747,21 +767,25 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
             BW_TRY(bw_v0(b, mode, w.V0in[l], s), "ofv_backward: stage input field");
         }
         a.Vout = w.Vst[sidx];
-        if (w.Sst[sidx]) {  // keep the window sums for the solve adjoint
+        cudaError_t e;
+        if (block) {  // keep the window sums for the solve adjoint
             a.s_out = w.Sst[sidx];
             a.s_plane = (size_t)h->Hs[l] * h->pitch[l];
             a.s_pitch = h->pitch[l];
+            const CUtensorMap *tm[2] = {&h->tmap[0][l], &h->tmap[1][l]};
+            const bool use = h->tma_ok[l] && h->tma_err_d;
+            e = launch_iter_block(&a, 1, p.storage, stage_mode(sidx), s, use ? tm : nullptr, h->tma_err_d, 0, 0,
+                                  tile_shape_of(p), sidx == 0 ? 1 : 2);
+        } else {
+            e = launch_iter_fused(a, p.storage, V0_SAME, s);
         }
-        cudaError_t e = block_supports(p.kernel_radius) ? launch_iter_block(&a, 1, p.storage, V0_SAME, s)
-                                                        : launch_iter_fused(a, p.storage, V0_SAME, s);
         BW_TRY(e, "ofv_backward: forward iteration");
     }
 
     // reverse
-    for (int l = 0; l < L; ++l) {
-        BW_TRY(cudaMemsetAsync(w.gP1[l], 0, (size_t)h->Hs[l] * h->pitch[l] * sizeof(float), s), "ofv_backward: memset");
-        BW_TRY(cudaMemsetAsync(w.gP2[l], 0, (size_t)h->Hs[l] * h->pitch[l] * sizeof(float), s), "ofv_backward: memset");
-    }
+    // the image gradients of all levels lie one after another
+    BW_TRY(cudaMemsetAsync(w.gP1[0], 0, reinterpret_cast<char *>(w.gw_scratch) - reinterpret_cast<char *>(w.gP1[0]), s),
+           "ofv_backward: memset");
     BW_TRY(bw_pack(gu, gv, h->H, h->W, w.gV, h->pitch[0], s), "ofv_backward: packing dL/dV");
     float2 *gV = w.gV, *gV0 = w.gV0;
     for (int sidx = S - 1; sidx >= 0; --sidx) {
@@ -771,7 +795,7 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
         A.pitch = B.pitch = Sk.pitch = h->pitch[l];
         if (w.Sst[sidx])
             for (int c = 0; c < 5; ++c) Sk.p[c] = w.Sst[sidx] + c * (size_t)h->Hs[l] * h->pitch[l];
-        BW_TRY(bw_stage(a, p.storage, Sk, A, B, gV, gV0, sidx == 0, w.gP1[l], w.gP2[l], h->pitch[l], s),
+        BW_TRY(bw_stage(a, stage_mode(sidx), p.storage, Sk, A, B, gV, gV0, sidx == 0, w.gP1[l], w.gP2[l], h->pitch[l], s),
                "ofv_backward: stage adjoint");
         if (sidx == 0) break;
         if (t > 0) {

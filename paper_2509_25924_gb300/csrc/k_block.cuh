@@ -872,7 +872,7 @@ struct QueueParams {
 // only; the batched launch has ITER_BOX and ITER_VAR)
 enum IterKind : int {
     ITER_BOX = 0,   // uniform box window (k_walk.cuh)
-    ITER_KEEP = 1,  // the same, keeping the window sums for the reverse mode
+    ITER_KEEP = 1,  // ITER_CHAIN keeping the window sums, for the reverse mode
     ITER_VAR = 2,   // estimator variants: Gaussian window, increment form, region mask
     ITER_CHAIN = 3  // ITER_BOX in a chain of launches that overlap their ends (a kernel of its own: the
                     // two instructions cost a stream of plain launches 2 %)

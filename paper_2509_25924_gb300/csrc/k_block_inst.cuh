@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(IterShape<T, KS, KIND>::NT, IterShape<T, KS, K
         block_tile<T, KS, false>(prm.a[z], prm.mode, blockIdx.x, prm.row0 / IterShape<T, KS, KIND>::TY + blockIdx.y, smem_f4,
                                  tm1, tm2, prm.err, s_bar);
     } else {
-        walk_tile<T, typename IterShape<T, KS, KIND>::WS, false, KIND == ITER_KEEP, KIND == ITER_CHAIN>(
+        walk_tile<T, typename IterShape<T, KS, KIND>::WS, false, KIND == ITER_KEEP, KIND != ITER_BOX>(
             prm.a[z], prm.mode, blockIdx.x, blockIdx.y, prm.row0, prm.row1, smem_f4, tm1, tm2, prm.err, s_bar,
             prm.overlap == 2);
     }
@@ -167,7 +167,7 @@ cudaError_t run_block(const BlockParams &p, dim3 grid, int dev, cudaStream_t s)
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) granted[dev] = smem;
     }
-    return launch_after(KIND == ITER_CHAIN, kern, grid, dim3(IterShape<T, KS, KIND>::NT), smem, s, p);
+    return launch_after(KIND == ITER_CHAIN || KIND == ITER_KEEP, kern, grid, dim3(IterShape<T, KS, KIND>::NT), smem, s, p);
 }
 
 // KS = kr + 16 shape for the radii and shapes instantiated here: every

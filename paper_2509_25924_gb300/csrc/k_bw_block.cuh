@@ -27,6 +27,8 @@ __global__ void __launch_bounds__(BlockShape<KR>::NT, BlockShape<KR>::MINB) k_bw
 {
     using BS = BlockShape<KR>;
     constexpr int TS = BS::TS, NT = BS::NT, RW = BS::RW, RWP = BS::RWP, PLANE = RW * RWP;
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(128) float4 smem_f4[];
     float *pl = reinterpret_cast<float *>(smem_f4);
     const int tid = threadIdx.x;
@@ -74,8 +76,8 @@ cudaError_t run_bw_box_tile(Planes5 in, Planes5 out, int H, int W, cudaStream_t 
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) granted[dev] = true;
     }
-    k_bw_box_tile<KR><<<dim3((W + BS::TS - 1) / BS::TS, (H + BS::TS - 1) / BS::TS), BS::NT, smem, s>>>(in, out, H, W);
-    return cudaGetLastError();
+    return launch_after(true, k_bw_box_tile<KR>, dim3((W + BS::TS - 1) / BS::TS, (H + BS::TS - 1) / BS::TS), dim3(BS::NT),
+                        smem, s, in, out, H, W);
 }
 
 }  // namespace ofv

@@ -27,7 +27,7 @@ constexpr int kBwRows = 8;  // rows a warp walks
 
 // GV0: the gradient of V0 is wanted (not at the first stage).
 template <typename T, bool GV0, typename General>
-__device__ __forceinline__ void bw_samples_walk(const IterArgs &a, const Planes5 &gq, float2 *gV0, float *gP1,
+__device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, const Planes5 &gq, float2 *gV0, float *gP1,
                                                 float *gP2, int gpitch, const General &general)
 {
     const int lane = threadIdx.x & 31;
@@ -88,7 +88,7 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, const Planes5
     auto fetch = [&](int y) {  // rows below the image repeat its last (and are not used)
         const int yc = min(y, H - 1);
         In in;
-        in.V0 = __ldg(a.V0 + (int64_t)yc * a.vpitch + xc);
+        in.V0 = fetch_v0_rt<false>(a, mode, xc, yc);
         const int64_t o = (int64_t)yc * gq.pitch + xc;
 #pragma unroll
         for (int c = 0; c < 5; ++c) in.q[c] = __ldg(gq.p[c] + o);
