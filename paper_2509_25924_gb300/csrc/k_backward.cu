@@ -243,88 +243,161 @@ __global__ void __launch_bounds__(128, 4) k_bw_samples_walk(const __grid_constan
     });
 }
 
-// Transpose of the x2 up-sampling: scatter 2 * w * gV0(fine) to the coarse
-// taps (gc zeroed beforehand).
+// Transpose of the x2 up-sampling, gathered: coarse pixel c takes from the
+// fine pixels 2c (weight 1), 2c - 1 and 2c + 1 (1/2; 1 where 2c + 1 has both
+// its taps on the last coarse pixel) of each axis.
 __global__ void k_bw_upsample_T(const float2 *gV0, int vpitch, int H, int W, float2 *gc, int cpitch, int Hc, int Wc)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= W || y >= H) return;
-    const float2 g = gV0[(int64_t)y * vpitch + x];
-    const int cx = x >> 1, cy = y >> 1;
-    const float fx = (x & 1) ? 0.5f : 0.f, fy = (y & 1) ? 0.5f : 0.f;
-    const int xa = min(cx, Wc - 1), xb = min(cx + 1, Wc - 1), ya = min(cy, Hc - 1), yb = min(cy + 1, Hc - 1);
-    const float w[4] = {(1.f - fx) * (1.f - fy), fx * (1.f - fy), (1.f - fx) * fy, fx * fy};
-    const int ty[4] = {ya, ya, yb, yb}, tx[4] = {xa, xb, xa, xb};
+    const int cx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int cy = blockIdx.y * blockDim.y + threadIdx.y;
+    if (cx >= Wc || cy >= Hc) return;
+    float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (w[k] == 0.f) continue;
-        float *p = reinterpret_cast<float *>(gc + (int64_t)ty[k] * cpitch + tx[k]);
-        atomicAdd(p, 2.f * w[k] * g.x);
-        atomicAdd(p + 1, 2.f * w[k] * g.y);
+    for (int dy = -1; dy <= 1; ++dy) {
+        const int y = 2 * cy + dy;
+        if (y < 0 || y >= H) continue;
+        const float wy = dy == 0 || (dy == 1 && cy == Hc - 1) ? 1.f : 0.5f;
+#pragma unroll
+        for (int dx = -1; dx <= 1; ++dx) {
+            const int x = 2 * cx + dx;
+            if (x < 0 || x >= W) continue;
+            const float w = 2.f * wy * (dx == 0 || (dx == 1 && cx == Wc - 1) ? 1.f : 0.5f);
+            const float2 g = __ldg(gV0 + (int64_t)y * vpitch + x);
+            s.x = fmaf(w, g.x, s.x);
+            s.y = fmaf(w, g.y, s.y);
+        }
     }
+    gc[(int64_t)cy * cpitch + cx] = s;
 }
 
-// Transpose of one pyramid reduction: level l+1 gradient (Hc x Wc) added
-// into level l (H x W), both dense with their pitches.
-__global__ void k_bw_reduce_T(const float *gc, int cpitch, int Hc, int Wc, float *g, int pitch, int H, int W)
+// Weight with which pixel i of n takes from coarse pixel c in the transpose
+// of the 5-tap reduction along one axis (taps outside clamp to the edge).
+__device__ __forceinline__ float reduce_weight(int i, int c, int n, int nc)
+{
+    if (c < 0 || c >= nc) return 0.f;
+    const float k[5] = {0.0625f, 0.25f, 0.375f, 0.25f, 0.0625f};
+    float w = 0.f;
+#pragma unroll
+    for (int a = 0; a < 5; ++a)
+        if (clampi(2 * c + a - 2, 0, n - 1) == i) w += k[a];
+    return w;
+}
+
+// Transpose of one pyramid reduction, gathered: level l+1 gradient (Hc x Wc)
+// added into level l (H x W), both dense with their pitches; blockIdx.z
+// selects the frame.  A pixel takes from the coarse pixels within one of its
+// half, the border's clamped taps included.
+__global__ void k_bw_reduce_T(const float *gc0, const float *gc1, int cpitch, int Hc, int Wc, float *g0, float *g1,
+                              int pitch, int H, int W)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= Hc || j >= Wc) return;
-    const float c[5] = {0.0625f, 0.25f, 0.375f, 0.25f, 0.0625f};
-    const float v = gc[(int64_t)i * cpitch + j];
-    if (v == 0.f) return;
+    if (i >= H || j >= W) return;
+    const float *gc = blockIdx.z ? gc1 : gc0;
+    float *g = (blockIdx.z ? g1 : g0) + (int64_t)i * pitch + j;
+    const int ci = i >> 1, cj = j >> 1;
+    float wx[3];
 #pragma unroll
-    for (int a = 0; a < 5; ++a)
+    for (int b = 0; b < 3; ++b) wx[b] = reduce_weight(j, cj + b - 1, W, Wc);
+    float s = 0.f;
 #pragma unroll
-        for (int b = 0; b < 5; ++b)
-            atomicAdd(g + (int64_t)clampi(2 * i + a - 2, 0, H - 1) * pitch + clampi(2 * j + b - 2, 0, W - 1),
-                      c[a] * c[b] * v);
+    for (int a = 0; a < 3; ++a) {
+        const float wy = reduce_weight(i, ci + a - 1, H, Hc);
+        if (wy == 0.f) continue;
+        const float *row = gc + (int64_t)(ci + a - 1) * cpitch;
+        float r = 0.f;
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            if (wx[b] != 0.f) r = fmaf(wx[b], __ldg(row + cj + b - 1), r);
+        s = fmaf(wy, r, s);
+    }
+    *g += s;
 }
 
-// Pre-filter transpose and weight gradient, then the input scaling:
-// gI(src) += w[a][b] * gJ(i,j) for src = clamp(i+a, j+b); gw[a][b] +=
-// gJ(i,j) * I(src).  The frame values I come from the raw input (scaled).
 template <typename TI>
 __device__ __forceinline__ float ld_raw(const TI *p) { return (float)__ldg(p); }
 
-template <typename TI>
-__global__ void k_bw_prefilter(const float *gJ, int pitch, int H, int W, const TI *raw, float scale, const float *w25,
-                               float *gI, float *gw)
+// Pixels i' of n whose pre-filter tap a reads pixel i (clamp-to-edge).
+__device__ __forceinline__ void tap_sources(int i, int a, int n, int &lo, int &hi)
 {
-    __shared__ float sw[25][8];
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    const int lane = threadIdx.x + threadIdx.y * blockDim.x;
+    lo = i == n - 1 ? n + 1 - a : i - a + 2;
+    hi = i == 0 ? 2 - a : i - a + 2;
+    if (i == n - 1) hi = max(hi, n - 1);
+    if (i == 0) lo = min(lo, 0);
+    lo = max(lo, 0);
+    hi = min(hi, n - 1);
+}
+
+// Pre-filter transpose and weight gradient, then the input scaling, gathered:
+// gI(p) = scale sum of w[a][b] gJ(k) over the pixels k whose tap (a, b) reads
+// p, gw[a][b] = sum of gJ(k) I(k + (a, b)) (clamp-to-edge).  The frame values
+// I come from the raw input (scaled).  A CTA of 32 x 8 threads takes a 32 x 32
+// block of gJ and of the frame with two pixels around it into shared memory;
+// the weight gradient is reduced once per CTA.  (The scattered form made 25
+// global atomics a pixel: 34 us a frame of 1 Mp.)
+template <typename TI>
+__global__ void __launch_bounds__(256) k_bw_prefilter(const float *gJ, int pitch, int H, int W, const TI *raw,
+                                                      float scale, const float *w25, float *gI, float *gw)
+{
+    __shared__ float sg[36][37], si[36][37];
+    __shared__ float sw[25][8], wt[25];
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    if (tid < 25) wt[tid] = __ldg(w25 + tid);
+    for (int t = tid; t < 36 * 36; t += 256) {
+        const int r = t / 36, c = t - r * 36;
+        const int y = by + r - 2, x = bx + c - 2;
+        const bool in = y >= 0 && y < H && x >= 0 && x < W;
+        sg[r][c] = in ? __ldg(gJ + (int64_t)y * pitch + x) : 0.f;
+        si[r][c] = ld_raw(raw + (int64_t)clampi(y, 0, H - 1) * W + clampi(x, 0, W - 1)) * scale;
+    }
+    __syncthreads();
     float acc[25];
 #pragma unroll
     for (int k = 0; k < 25; ++k) acc[k] = 0.f;
-    if (i < H && j < W) {
-        const float g = gJ[(int64_t)i * pitch + j];
-        if (g != 0.f) {
+    const int j = bx + threadIdx.x;
+#pragma unroll 1
+    for (int ly = threadIdx.y; ly < 32; ly += 8) {
+        const int i = by + ly;
+        if (i >= H || j >= W) break;
+        float s = 0.f;
+        if (i > 0 && i < H - 1 && j > 0 && j < W - 1) {  // taps outside the image are zero in sg
 #pragma unroll
             for (int a = 0; a < 5; ++a)
 #pragma unroll
+                for (int b = 0; b < 5; ++b) s = fmaf(wt[a * 5 + b], sg[ly + 4 - a][threadIdx.x + 4 - b], s);
+        } else {
+            for (int a = 0; a < 5; ++a) {
+                int y0, y1;
+                tap_sources(i, a, H, y0, y1);
                 for (int b = 0; b < 5; ++b) {
-                    const int64_t src = (int64_t)clampi(i + a - 2, 0, H - 1) * W + clampi(j + b - 2, 0, W - 1);
-                    atomicAdd(gI + src, __ldg(w25 + a * 5 + b) * g * scale);
-                    acc[a * 5 + b] = g * ld_raw(raw + src) * scale;
+                    int x0, x1;
+                    tap_sources(j, b, W, x0, x1);
+                    for (int y = y0; y <= y1; ++y)
+                        for (int x = x0; x <= x1; ++x)
+                            s = fmaf(wt[a * 5 + b], sg[y - by + 2][x - bx + 2], s);  // within two pixels
                 }
+            }
         }
+        gI[(int64_t)i * W + j] = s * scale;
+        const float g = sg[ly + 2][threadIdx.x + 2];
+#pragma unroll
+        for (int a = 0; a < 5; ++a)
+#pragma unroll
+            for (int b = 0; b < 5; ++b) acc[a * 5 + b] = fmaf(g, si[ly + a][threadIdx.x + b], acc[a * 5 + b]);
     }
-    // block reduction of the weight gradient: warp shuffles, then one atomic per warp
+    // block reduction of the weight gradient: warp shuffles, then one atomic per CTA and weight
 #pragma unroll
     for (int k = 0; k < 25; ++k) {
         float v = acc[k];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((lane & 31) == 0) sw[k][lane >> 5] = v;
+        if (threadIdx.x == 0) sw[k][threadIdx.y] = v;
     }
     __syncthreads();
-    if (lane < 25) {
+    if (tid < 25) {
         float s = 0.f;
-        for (int k = 0; k < (int)(blockDim.x * blockDim.y + 31) / 32; ++k) s += sw[lane][k];
-        atomicAdd(gw + lane, s);
+        for (int k = 0; k < 8; ++k) s += sw[tid][k];
+        atomicAdd(gw + tid, s);
     }
 }
 
@@ -379,63 +452,60 @@ __global__ void k_bw_norm_stats(const TI *raw, float scale, int H, int W, int nr
     J[k] = (ld_raw(raw + k) * scale - m) / sv;
 }
 
-// alpha = a / (s n), beta = a J / (s^2 n), gamma = beta mu.
-__global__ void k_bw_norm_coef(const float *a, const float *J, const float *mu, const float *sd, int H, int W, int nr,
-                               float *alpha, float *beta, float *gamma)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= H || j >= W) return;
-    const int64_t k = (int64_t)i * W + j;
-    const float sn = sd[k] * (float)box_count(i, j, H, W, nr);
-    const float al = a[k] / sn;
-    const float be = al * J[k] / sd[k];
-    alpha[k] = al;
-    beta[k] = be;
-    gamma[k] = be * mu[k];
-}
-
-// Truncated box sums of radius nr of three planes along rows (dir 0) or
-// columns (dir 1).
-__global__ void k_bw_box3(const float *x0, const float *x1, const float *x2, int H, int W, int nr, int dir, float *y0,
-                          float *y1, float *y2)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= H || j >= W) return;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    if (dir == 0) {
-        const int64_t r = (int64_t)i * W;
-        for (int jj = max(j - nr, 0); jj <= min(j + nr, W - 1); ++jj) {
-            s0 += x0[r + jj];
-            s1 += x1[r + jj];
-            s2 += x2[r + jj];
-        }
-    } else {
-        for (int ii = max(i - nr, 0); ii <= min(i + nr, H - 1); ++ii) {
-            const int64_t o = (int64_t)ii * W + j;
-            s0 += x0[o];
-            s1 += x1[o];
-            s2 += x2[o];
-        }
-    }
-    const int64_t k = (int64_t)i * W + j;
-    y0[k] = s0;
-    y1[k] = s1;
-    y2[k] = s2;
-}
-
+// The rest of the adjoint: alpha = a / (s n), beta = a J / (s^2 n) and
+// beta mu over a 32 x 32 block and its NR halo in shared memory, their
+// truncated box sums (rows, then columns), and
 // dL/draw = scale (a/s - A - I B + C), I = raw * scale.
 template <typename TI>
-__global__ void k_bw_norm_out(const float *a, const float *sd, const TI *raw, float scale, const float *A,
-                              const float *B, const float *C, int H, int W, float *gI)
+__global__ void __launch_bounds__(256) k_bw_norm_out(const float *a, const float *J, const float *mu, const float *sd,
+                                                     const TI *raw, float scale, int H, int W, int nr, float *gI)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= H || j >= W) return;
-    const int64_t k = (int64_t)i * W + j;
-    const float I = ld_raw(raw + k) * scale;
-    gI[k] = scale * (a[k] / sd[k] - A[k] - I * B[k] + C[k]);
+    extern __shared__ float sm[];  // three planes of TW x TW, then of TW x 32 row sums
+    const int TW = 32 + 2 * nr, K = 2 * nr + 1;
+    float *pl = sm, *rs = sm + 3 * TW * TW;
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    for (int t = tid; t < TW * TW; t += 256) {
+        const int r = t / TW, c = t - r * TW;
+        const int i = by + r - nr, j = bx + c - nr;
+        float al = 0.f, be = 0.f, ga = 0.f;
+        if (i >= 0 && i < H && j >= 0 && j < W) {
+            const int64_t k = (int64_t)i * W + j;
+            const float s = __ldg(sd + k);
+            al = __ldg(a + k) / (s * (float)box_count(i, j, H, W, nr));
+            be = al * __ldg(J + k) / s;
+            ga = be * __ldg(mu + k);
+        }
+        pl[t] = al;
+        pl[TW * TW + t] = be;
+        pl[2 * TW * TW + t] = ga;
+    }
+    __syncthreads();
+    for (int t = tid; t < 3 * TW * 32; t += 256) {  // (plane, row) in order, 32 columns each
+        const float *row = pl + (t >> 5) * TW + (t & 31);
+        float v = 0.f;
+        for (int k = 0; k < K; ++k) v += row[k];
+        rs[t] = v;
+    }
+    __syncthreads();
+    const int j = bx + threadIdx.x;
+    if (j >= W) return;
+#pragma unroll 1
+    for (int ly = threadIdx.y; ly < 32; ly += 8) {
+        const int i = by + ly;
+        if (i >= H) break;
+        float S[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float *col = rs + (c * TW + ly) * 32 + threadIdx.x;
+            float v = 0.f;
+            for (int k = 0; k < K; ++k) v += col[k * 32];
+            S[c] = v;
+        }
+        const int64_t k = (int64_t)i * W + j;
+        const float I = ld_raw(raw + k) * scale;
+        gI[k] = scale * (__ldg(a + k) / __ldg(sd + k) - S[0] - I * S[1] + S[2]);
+    }
 }
 
 // Dense planar (gu, gv) into an interleaved field of pitch vpitch.
@@ -530,38 +600,47 @@ cudaError_t bw_stage(const IterArgs &a, int mode, int store, Planes5 Sk, Planes5
 cudaError_t bw_upsample_T(const float2 *gV0, int vpitch, int H, int W, float2 *gc, int cpitch, int Hc, int Wc,
                           cudaStream_t s)
 {
-    k_bw_upsample_T<<<grid2(W, H), dim3(32, 8), 0, s>>>(gV0, vpitch, H, W, gc, cpitch, Hc, Wc);
+    k_bw_upsample_T<<<grid2(Wc, Hc), dim3(32, 8), 0, s>>>(gV0, vpitch, H, W, gc, cpitch, Hc, Wc);
     return cudaGetLastError();
 }
 
-cudaError_t bw_reduce_T(const float *gc, int cpitch, int Hc, int Wc, float *g, int pitch, int H, int W, cudaStream_t s)
+cudaError_t bw_reduce_T(const float *gc0, const float *gc1, int cpitch, int Hc, int Wc, float *g0, float *g1, int pitch,
+                        int H, int W, cudaStream_t s)
 {
-    k_bw_reduce_T<<<grid2(Wc, Hc), dim3(32, 8), 0, s>>>(gc, cpitch, Hc, Wc, g, pitch, H, W);
+    dim3 g = grid2(W, H);
+    g.z = 2;
+    k_bw_reduce_T<<<g, dim3(32, 8), 0, s>>>(gc0, gc1, cpitch, Hc, Wc, g0, g1, pitch, H, W);
     return cudaGetLastError();
 }
 
 // Reverse of ingest with local normalization: J (pyramid level 0) = pre-filter
 // (optional) of the normalized frame N; gJ -> gN (pre-filter transpose, weight
-// gradient against N) -> gI through the normalization adjoint.  t[0..9]:
+// gradient against N) -> gI through the normalization adjoint.  t[0..3]:
 // dense H x W scratch planes.
 template <typename TI>
 cudaError_t bw_input_norm_t(const float *gJ, int pitch, int H, int W, const TI *raw, float scale, int nr, float eps_n,
                             const float *w25, int prefilter, float *gI, float *gw, float *const *t, cudaStream_t s)
 {
-    const dim3 g = grid2(W, H), b(32, 8);
+    const dim3 g = grid2(W, H), b(32, 8), gt((W + 31) / 32, (H + 31) / 32);
+    const int TW = 32 + 2 * nr;
     float *N = t[0], *mu = t[1], *sd = t[2], *gN = t[3];
     k_bw_norm_stats<TI><<<g, b, 0, s>>>(raw, scale, H, W, nr, eps_n, N, mu, sd);
     if (prefilter) {
-        cudaError_t e = cudaMemsetAsync(gN, 0, (size_t)H * W * sizeof(float), s);
-        if (e != cudaSuccess) return e;
-        k_bw_prefilter<float><<<g, b, 0, s>>>(gJ, pitch, H, W, N, 1.f, w25, gN, gw);
+        k_bw_prefilter<float><<<gt, b, 0, s>>>(gJ, pitch, H, W, N, 1.f, w25, gN, gw);
     } else {
         k_bw_copy_scaled<<<g, b, 0, s>>>(gJ, pitch, H, W, 1.f, gN);
     }
-    k_bw_norm_coef<<<g, b, 0, s>>>(gN, N, mu, sd, H, W, nr, t[4], t[5], t[6]);
-    k_bw_box3<<<g, b, 0, s>>>(t[4], t[5], t[6], H, W, nr, 0, t[7], t[8], t[9]);
-    k_bw_box3<<<g, b, 0, s>>>(t[7], t[8], t[9], H, W, nr, 1, t[4], t[5], t[6]);
-    k_bw_norm_out<TI><<<g, b, 0, s>>>(gN, sd, raw, scale, t[4], t[5], t[6], H, W, gI);
+    const size_t smem = sizeof(float) * 3 * TW * (TW + 32);  // 72 KB at NR 16
+    static bool granted[64];  // shared-memory opt-in done, per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && (dev < 0 || dev >= 64 || !granted[dev])) {
+        e = cudaFuncSetAttribute(k_bw_norm_out<TI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(float) * 3 * 64 * 96));
+        if (e == cudaSuccess && dev >= 0 && dev < 64) granted[dev] = true;
+    }
+    if (e != cudaSuccess) return e;
+    k_bw_norm_out<TI><<<gt, b, smem, s>>>(gN, N, mu, sd, raw, scale, H, W, nr, gI);
     return cudaGetLastError();
 }
 
@@ -587,10 +666,11 @@ cudaError_t bw_input(const float *gJ, int pitch, int H, int W, const void *raw, 
         k_bw_copy_scaled<<<g, b, 0, s>>>(gJ, pitch, H, W, scale, gI);
         return cudaGetLastError();
     }
+    const dim3 gp((W + 31) / 32, (H + 31) / 32);
     switch (in_type) {
-    case IN_U8: k_bw_prefilter<uint8_t><<<g, b, 0, s>>>(gJ, pitch, H, W, static_cast<const uint8_t *>(raw), scale, w25, gI, gw); break;
-    case IN_U16: k_bw_prefilter<uint16_t><<<g, b, 0, s>>>(gJ, pitch, H, W, static_cast<const uint16_t *>(raw), scale, w25, gI, gw); break;
-    default: k_bw_prefilter<float><<<g, b, 0, s>>>(gJ, pitch, H, W, static_cast<const float *>(raw), scale, w25, gI, gw); break;
+    case IN_U8: k_bw_prefilter<uint8_t><<<gp, b, 0, s>>>(gJ, pitch, H, W, static_cast<const uint8_t *>(raw), scale, w25, gI, gw); break;
+    case IN_U16: k_bw_prefilter<uint16_t><<<gp, b, 0, s>>>(gJ, pitch, H, W, static_cast<const uint16_t *>(raw), scale, w25, gI, gw); break;
+    default: k_bw_prefilter<float><<<gp, b, 0, s>>>(gJ, pitch, H, W, static_cast<const float *>(raw), scale, w25, gI, gw); break;
     }
     return cudaGetLastError();
 }
@@ -803,26 +883,18 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
             gV = gV0;
             gV0 = tmp;
         } else {
-            BW_TRY(cudaMemsetAsync(gV, 0, (size_t)h->Hs[l + 1] * h->pitch[l + 1] * sizeof(float2), s),
-                   "ofv_backward: memset");
             BW_TRY(bw_upsample_T(gV0, h->pitch[l], h->Hs[l], h->Ws[l], gV, h->pitch[l + 1], h->Hs[l + 1], h->Ws[l + 1], s),
                    "ofv_backward: up-sampling adjoint");
         }
     }
     for (int l = L - 1; l >= 1; --l) {
-        BW_TRY(bw_reduce_T(w.gP1[l], h->pitch[l], h->Hs[l], h->Ws[l], w.gP1[l - 1], h->pitch[l - 1], h->Hs[l - 1],
-                           h->Ws[l - 1], s),
-               "ofv_backward: reduce adjoint");
-        BW_TRY(bw_reduce_T(w.gP2[l], h->pitch[l], h->Hs[l], h->Ws[l], w.gP2[l - 1], h->pitch[l - 1], h->Hs[l - 1],
-                           h->Ws[l - 1], s),
+        BW_TRY(bw_reduce_T(w.gP1[l], w.gP2[l], h->pitch[l], h->Hs[l], h->Ws[l], w.gP1[l - 1], w.gP2[l - 1],
+                           h->pitch[l - 1], h->Hs[l - 1], h->Ws[l - 1], s),
                "ofv_backward: reduce adjoint");
     }
     const float scale = p.input == OFV_IN_F32 ? 1.0f : 1.0f / (float)((1u << p.bit_depth) - 1u);
     float *gw = gw25 ? gw25 : w.gw_scratch;
-    const size_t nbytes = (size_t)h->H * h->W * sizeof(float);
     if (p.prefilter) {
-        BW_TRY(cudaMemsetAsync(gI1, 0, nbytes, s), "ofv_backward: memset");
-        BW_TRY(cudaMemsetAsync(gI2, 0, nbytes, s), "ofv_backward: memset");
         BW_TRY(cudaMemsetAsync(gw, 0, 25 * sizeof(float), s), "ofv_backward: memset");
     } else if (gw25) {
         BW_TRY(cudaMemsetAsync(gw25, 0, 25 * sizeof(float), s), "ofv_backward: memset");
