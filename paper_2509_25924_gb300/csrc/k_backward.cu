@@ -229,16 +229,16 @@ __device__ __noinline__ void samples_adjoint_general(const IterArgs *a, int mode
 }
 
 // The same with the taps and the gradients of a walk down the columns in
-// registers (k_bw_walk.cuh); four warps per CTA, 32 columns x kBwRows rows
+// registers (k_bw_walk.cuh); four warps per CTA, 32 columns x NROW rows
 // each.
-template <typename T, bool GV0>
+template <typename T, bool GV0, int NROW>
 __global__ void __launch_bounds__(128, 4) k_bw_samples_walk(const __grid_constant__ IterArgs a, int mode,
                                                             const __grid_constant__ Planes5 gprod, float2 *gV0,
                                                             float *gP1, float *gP2, int gpitch)
 {
     pdl_wait();
     pdl_trigger();
-    bw_samples_walk<T, GV0>(a, mode, gprod, gV0, gP1, gP2, gpitch, [&](int x, int y) {
+    bw_samples_walk<T, GV0, NROW>(a, mode, gprod, gV0, gP1, gP2, gpitch, [&](int x, int y) {
         samples_adjoint_general<T>(&a, mode, &gprod, gV0, x, y, gP1, gP2, gpitch);
     });
 }
@@ -553,9 +553,12 @@ template <typename T>
 cudaError_t samples_walk(const IterArgs &a, int mode, const Planes5 &A, float2 *gV0, bool first, float *gP1, float *gP2,
                          int gpitch, cudaStream_t s)
 {
-    const dim3 g((a.W + 31) / 32, (a.H + 4 * kBwRows - 1) / (4 * kBwRows));
-    return launch_after(true, first ? k_bw_samples_walk<T, false> : k_bw_samples_walk<T, true>, g, dim3(128), 0, s, a, mode,
-                        A, gV0, gP1, gP2, gpitch);
+    const int rows = bw_rows(a.H, a.W);
+    const dim3 g((a.W + 31) / 32, (a.H + 4 * rows - 1) / (4 * rows));
+    auto kern = rows == kBwRows
+                    ? (first ? k_bw_samples_walk<T, false, kBwRows> : k_bw_samples_walk<T, true, kBwRows>)
+                    : (first ? k_bw_samples_walk<T, false, kBwRowsSmall> : k_bw_samples_walk<T, true, kBwRowsSmall>);
+    return launch_after(true, kern, g, dim3(128), 0, s, a, mode, A, gV0, gP1, gP2, gpitch);
 }
 }  // namespace
 

@@ -23,16 +23,23 @@
 
 namespace ofv {
 
-constexpr int kBwRows = 8;  // rows a warp walks
+// Rows a warp walks: 8, or 4 where the 8-row warps of a level would all be
+// resident at once (152 SMs x 16 warps), so that only the length of a walk
+// counts.
+constexpr int kBwRows = 8, kBwRowsSmall = 4;
+inline int bw_rows(int H, int W)
+{
+    return (long long)((W + 31) / 32) * ((H + kBwRows - 1) / kBwRows) <= 152 * 16 ? kBwRowsSmall : kBwRows;
+}
 
 // GV0: the gradient of V0 is wanted (not at the first stage).
-template <typename T, bool GV0, typename General>
+template <typename T, bool GV0, int NROW, typename General>
 __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, const Planes5 &gq, float2 *gV0, float *gP1,
                                                 float *gP2, int gpitch, const General &general)
 {
     const int lane = threadIdx.x & 31;
     const int x = blockIdx.x * 32 + lane;
-    const int y0 = (blockIdx.y * (blockDim.x / 32) + (threadIdx.x >> 5)) * kBwRows;
+    const int y0 = (blockIdx.y * (blockDim.x / 32) + (threadIdx.x >> 5)) * NROW;
     const int H = a.H, W = a.W, pitch = a.pitch;
     if (y0 >= H) return;
     const T *P1 = static_cast<const T *>(a.P1), *P2 = static_cast<const T *>(a.P2);
@@ -81,7 +88,7 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
     };
     // V0 and the products' gradients of a row, loaded a step ahead
     struct In {
-        float2 V0;
+        float2 V0, gV0;
         float q[5];
     };
     const int xc = min(x, W - 1);
@@ -89,6 +96,7 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
         const int yc = min(y, H - 1);
         In in;
         in.V0 = fetch_v0_rt<false>(a, mode, xc, yc);
+        if (GV0) in.gV0 = gV0[(int64_t)yc * a.vpitch + xc];
         const int64_t o = (int64_t)yc * gq.pitch + xc;
 #pragma unroll
         for (int c = 0; c < 5; ++c) in.q[c] = __ldg(gq.p[c] + o);
@@ -97,7 +105,7 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
     unsigned rest = 0;  // rows whose pixel needs the general form
     In nxt = fetch(y0);
 #pragma unroll 1
-    for (int ib = 0; ib < kBwRows; ib += 4) {
+    for (int ib = 0; ib < NROW; ib += 4) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             // a step past the image's last row has no pixel: what is left of
@@ -105,7 +113,7 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
             const int y = y0 + ib + j;
             const int s0 = j, s1 = (j + 1) & 3, s2 = (j + 2) & 3, s3 = (j + 3) & 3;
             const In cur = nxt;
-            if (ib + j + 1 < kBwRows) nxt = fetch(y + 1);
+            if (ib + j + 1 < NROW) nxt = fetch(y + 1);
             const float2 V0 = cur.V0;
             const float q0 = cur.q[0], q1 = cur.q[1], q2 = cur.q[2], q3 = cur.q[3], q4 = cur.q[4];
             int ix, iy;
@@ -160,11 +168,10 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
                     const float hx = gGx * (u1 - u0) + gGy * (Dv.y - Dv.x) - gr * (Pv.y - Pv.x);
                     const float hy = gGx * (wx * (dP.y - dF.x) + fx * (dF.y - dP.x)) + gGy * (wx * dD.x + fx * dD.y) -
                                      gr * (wx * dP.x + fx * dP.y);
-                    float2 *gp = gV0 + (int64_t)y * a.vpitch + x;
-                    float2 g = *gp;
+                    float2 g = cur.gV0;
                     g.x += Gx * gr + 0.5f * hx;
                     g.y += Gy * gr + 0.5f * hy;
-                    *gp = g;
+                    gV0[(int64_t)y * a.vpitch + x] = g;
                 }
                 // Gx, Gy, It -> the rows' interpolations -> E
                 const float2 gPv = make_float2(-wx * gr - fx * gGx, -fx * gr + wx * gGx);
