@@ -868,8 +868,8 @@ struct QueueParams {
 // of iteration in k_block_{f32,f16,bf16}.cu (ITER_BOX) and
 // k_block_var_{f32,f16,bf16}.cu (ITER_KEEP and ITER_VAR) and
 // k_block_chain_{f32,f16,bf16}.cu (ITER_CHAIN).
-// shape: the tile shape v (ITER_KEEP and ITER_VAR have the default shape
-// only; the batched launch has ITER_BOX and ITER_VAR)
+// shape: the tile shape v (ITER_VAR has the default shape only, ITER_KEEP the
+// smaller one of radii 3 and 4; the batched launch has ITER_BOX and ITER_VAR)
 enum IterKind : int {
     ITER_BOX = 0,   // uniform box window (k_walk.cuh)
     ITER_KEEP = 1,  // ITER_CHAIN keeping the window sums, for the reverse mode

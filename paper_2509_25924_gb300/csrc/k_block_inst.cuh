@@ -172,11 +172,18 @@ cudaError_t run_block(const BlockParams &p, dim3 grid, int dev, cudaStream_t s)
 
 // KS = kr + 16 shape for the radii and shapes instantiated here: every
 // radius with its default shape; the alternative shapes without the
-// estimator variants.  0 when not instantiated.
+// estimator variants (keeping the window sums, of radii 3 and 4, whose small
+// levels take them).  0 when not instantiated.
+template <int KIND>
+constexpr bool has_alt(int kr)
+{
+    return KIND == ITER_BOX || KIND == ITER_CHAIN || (KIND == ITER_KEEP && (kr == 3 || kr == 4));
+}
 template <int KIND>
 constexpr int ks_of(int kr, int shape)
 {
-    return (kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1 || (KIND != ITER_BOX && KIND != ITER_CHAIN && shape != 0)) ? 0 : kr + 16 * shape;
+    return kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1 || (shape != 0 && !has_alt<KIND>(kr)) ? 0
+                                                                                                 : kr + 16 * shape;
 }
 
 #define OFV_KS_CASES(X)                                                                                    \
@@ -194,7 +201,7 @@ cudaError_t launch_block_t(const BlockParams &p, int kr, int npairs, cudaStream_
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
+        if constexpr (has_alt<KIND>((K) - 16)) { X##_BODY(K) } else { break; }
 #define OFV_BLOCK_CASE(K) case K: OFV_BLOCK_CASE_BODY(K)
 #define OFV_BLOCK_CASE_BODY(K)                                                                             \
     {                                                                                                      \
@@ -252,7 +259,7 @@ cudaError_t launch_queue_t(const QueueParams &q, int kr, cudaStream_t s, int sha
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
+        if constexpr (has_alt<KIND>((K) - 16)) { X##_BODY(K) } else { break; }
 #define OFV_QUEUE_CASE(K) case K: OFV_QUEUE_CASE_BODY(K)
 #define OFV_QUEUE_CASE_BODY(K) return run_queue<T, QKS(K), KIND>(q, dev, s);
     OFV_KS_CASES(OFV_QUEUE_CASE)
@@ -271,7 +278,7 @@ int queue_occupancy_t(int kr, int shape)
     switch (ks_of<KIND>(kr, shape)) {
 #define OFV_KS_ALT(X, K) \
     case K:              \
-        if constexpr (KIND == ITER_BOX || KIND == ITER_CHAIN) { X##_BODY(K) } else { break; }
+        if constexpr (has_alt<KIND>((K) - 16)) { X##_BODY(K) } else { break; }
 #define OFV_OCC_CASE(K) case K: OFV_OCC_CASE_BODY(K)
 #define OFV_OCC_CASE_BODY(K) return queue_occupancy_kr<T, QKS(K), KIND>();
     OFV_KS_CASES(OFV_OCC_CASE)

@@ -106,7 +106,7 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
         block_stage_box(store, a[0].kr, &c1, &r1, 0, true);
         if (c0 != c1 || r0 != r1) p.use_tma = 0;
     }
-    if ((kind == ITER_BOX || kind == ITER_CHAIN) && shape == 0 && npairs == 1 && walk_small_tiles(a[0].kr, a[0].W, p.row1 - row0)) shape = 1;
+    if (kind != ITER_VAR && shape == 0 && npairs == 1 && walk_small_tiles(a[0].kr, a[0].W, p.row1 - row0)) shape = 1;
     switch (store) {
     case ST_F16: return launch_kind<__half>(p, kind, a[0].kr, npairs, s, shape);
     case ST_BF16: return launch_kind<__nv_bfloat16>(p, kind, a[0].kr, npairs, s, shape);
