@@ -22,9 +22,9 @@ template <typename T, int KS> struct IterShape<T, KS, ITER_VAR> {
 // One tile per CTA; blockIdx.z selects the pair.
 //
 // ITER_BOX, 8 pairs of 1 Mp, level 0, FP32, KR 4, V0 from the previous
-// iteration (ncu): 17.2 M shared-memory wavefronts, 60.7 M warp instructions
-// (231 thread instructions per output), LSU data pipe 64 % of peak over the
-// launch and issue 50 %, 103 us; the one-pixel-per-thread form before it:
+// iteration (ncu): 17.1 M shared-memory wavefronts, 60.5 M warp instructions
+// (231 thread instructions per output), LSU data pipe 63 % of peak over the
+// launch and issue 49 %, 105 us; the one-pixel-per-thread form before it:
 // 23.2 M wavefronts, 99.6 M instructions, 121 us.  Shared-memory wavefronts
 // bound it: 24 taps and 5 stores a pixel of the halo tile became 11 + 5, and
 // the window sums 13 + 11 words per output instead of 35.  64 fields of a
