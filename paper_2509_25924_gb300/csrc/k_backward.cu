@@ -187,7 +187,7 @@ __device__ __forceinline__ void samples_adjoint_pixel(const IterArgs &a, int mod
 {
     const T *P1 = static_cast<const T *>(a.P1);
     const T *P2 = static_cast<const T *>(a.P2);
-    const float2 V0 = fetch_v0_rt<false>(a, mode, x, y);
+    const float2 V0 = fetch_v0_rt<LD_READ_ONLY>(a, mode, x, y);
     const float hx = 0.5f * V0.x, hy = 0.5f * V0.y;
     const Sample s1 = sample_level(P1, a.H, a.W, a.pitch, x, y, -hx, -hy);
     const Sample s2 = sample_level(P2, a.H, a.W, a.pitch, x, y, hx, hy);

@@ -223,18 +223,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, unsigned parity
     return false;
 }
 
-// Field load: through the read-only cache, or -- when the field was written
-// earlier in the same launch by other CTAs (persistent batched kernel) --
-// from L2 only, so no stale L1 line is read.
-template <bool COH>
+// Field loads: through the read-only cache; by ordinary loads where the launch
+// ahead wrote the field while this kernel was already resident (launch_after);
+// from L2 only where other CTAs of the same launch wrote it (the batched
+// kernel), so no stale L1 line is read.
+enum FieldLoad : int { LD_READ_ONLY = 0, LD_AFTER_WAIT = 1, LD_SAME_LAUNCH = 2 };
+template <int COH>
 __device__ __forceinline__ float2 ld_field(const float2 *p)
 {
-    return COH ? __ldcg(p) : __ldg(p);
+    return COH == LD_SAME_LAUNCH ? __ldcg(p) : COH == LD_AFTER_WAIT ? *p : __ldg(p);
 }
 
 // V0 at (x, y) with the mode chosen at run time (uniform per launch):
 // zero, the same-level field, or 2 * bilinear(coarse field, x/2, y/2).
-template <bool COH>
+template <int COH>
 __device__ __forceinline__ float2 fetch_v0_rt(const IterArgs &a, int mode, int x, int y)
 {
     if (mode == V0_SAME) return ld_field<COH>(a.V0 + (int64_t)y * a.vpitch + x);
@@ -257,7 +259,7 @@ __device__ __forceinline__ float2 fetch_v0_rt(const IterArgs &a, int mode, int x
 }
 
 // V0 with the mode fixed at compile time, for pixels inside the image.
-template <bool COH, int MODE>
+template <int COH, int MODE>
 __device__ __forceinline__ float2 fetch_v0_ct(const IterArgs &a, int x, int y)
 {
     if (MODE == V0_ZERO) return make_float2(0.f, 0.f);
@@ -454,7 +456,7 @@ __host__ __device__ constexpr int first_iter_of_band_up(int b)
 // With bars (TMA staging in three bands), the loop waits for band b just
 // before the first iteration that can touch it, so the first rows of
 // products overlap the copies of the later bands.
-template <typename T, int KR, bool COH, int MODE, int SP>
+template <typename T, int KR, int COH, int MODE, int SP>
 __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const T *__restrict__ st1,
                                                        const T *__restrict__ st2, int sx0, int sy0, int px0, int py0,
                                                        float *prod, uint64_t *bars, int *err)
@@ -620,7 +622,7 @@ __device__ __forceinline__ float recip_newton(float d)
 
 // Phase 4 of the forward iteration: the guarded 2x2 solve of pixel (gx, gy)
 // from its window sums S = (Sxx, Sxy, Syy, Sxr, Syr) and the store of V.
-template <bool COH>
+template <int COH>
 __device__ __forceinline__ void solve_store(const IterArgs &a, int mode, int gx, int gy, const float (&S)[5])
 {
     const float sxx = S[0], sxy = S[1], syy = S[2], sxr = S[3], syr = S[4];
@@ -651,7 +653,7 @@ __device__ __forceinline__ void solve_store(const IterArgs &a, int mode, int gx,
 // (increment form, Gaussian window, region mask).
 // TMA staging needs tensor maps tm1, tm2 of the two level images and NBAND
 // mbarriers tma_bars (shared memory).
-template <typename T, int KR, bool COH>
+template <typename T, int KR, int COH>
 __device__ __forceinline__ void block_tile(const IterArgs &a, int mode, int bx, int by, float4 *smem_f4,
                                            const CUtensorMap *tm1, const CUtensorMap *tm2, int *err,
                                            uint64_t *tma_bars)

@@ -39,10 +39,12 @@ __global__ void __launch_bounds__(IterShape<T, KS, KIND>::NT, IterShape<T, KS, K
     const int z = blockIdx.z;
     const CUtensorMap *tm1 = prm.use_tma ? &prm.tm[z][0] : nullptr, *tm2 = prm.use_tma ? &prm.tm[z][1] : nullptr;
     if constexpr (KIND == ITER_VAR) {
-        block_tile<T, KS, false>(prm.a[z], prm.mode, blockIdx.x, prm.row0 / IterShape<T, KS, KIND>::TY + blockIdx.y, smem_f4,
-                                 tm1, tm2, prm.err, s_bar);
+        block_tile<T, KS, LD_READ_ONLY>(prm.a[z], prm.mode, blockIdx.x,
+                                        prm.row0 / IterShape<T, KS, KIND>::TY + blockIdx.y, smem_f4, tm1, tm2, prm.err,
+                                        s_bar);
     } else {
-        walk_tile<T, typename IterShape<T, KS, KIND>::WS, false, KIND == ITER_KEEP, KIND != ITER_BOX>(
+        walk_tile<T, typename IterShape<T, KS, KIND>::WS, KIND == ITER_BOX ? LD_READ_ONLY : LD_AFTER_WAIT,
+                  KIND == ITER_KEEP, KIND != ITER_BOX>(
             prm.a[z], prm.mode, blockIdx.x, blockIdx.y, prm.row0, prm.row1, smem_f4, tm1, tm2, prm.err, s_bar,
             prm.overlap == 2);
     }
@@ -146,10 +148,10 @@ __global__ void __launch_bounds__(IterShape<T, KS, KIND>::NT, IterShape<T, KS, K
     if (s_fail) return;
     const CUtensorMap *tm1 = o.tm, *tm2 = o.tm ? o.tm + 1 : nullptr;
     if constexpr (VAR) {
-        block_tile<T, KS, true>(o.a, o.mode, o.bx, o.by, smem_f4, tm1, tm2, q.tma_err, s_bar);
+        block_tile<T, KS, LD_SAME_LAUNCH>(o.a, o.mode, o.bx, o.by, smem_f4, tm1, tm2, q.tma_err, s_bar);
     } else {
-        walk_tile<T, typename IterShape<T, KS, KIND>::WS, true, false, false>(o.a, o.mode, o.bx, o.by, 0, o.a.H, smem_f4, tm1,
-                                                                       tm2, q.tma_err, s_bar, false);
+        walk_tile<T, typename IterShape<T, KS, KIND>::WS, LD_SAME_LAUNCH, false, false>(
+            o.a, o.mode, o.bx, o.by, 0, o.a.H, smem_f4, tm1, tm2, q.tma_err, s_bar, false);
     }
     __threadfence();
     __syncthreads();

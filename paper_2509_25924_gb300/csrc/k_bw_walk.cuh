@@ -95,11 +95,11 @@ __device__ __forceinline__ void bw_samples_walk(const IterArgs &a, int mode, con
     auto fetch = [&](int y) {  // rows below the image repeat its last (and are not used)
         const int yc = min(y, H - 1);
         In in;
-        in.V0 = fetch_v0_rt<false>(a, mode, xc, yc);
+        in.V0 = fetch_v0_rt<LD_READ_ONLY>(a, mode, xc, yc);
         if (GV0) in.gV0 = gV0[(int64_t)yc * a.vpitch + xc];
         const int64_t o = (int64_t)yc * gq.pitch + xc;
 #pragma unroll
-        for (int c = 0; c < 5; ++c) in.q[c] = __ldg(gq.p[c] + o);
+        for (int c = 0; c < 5; ++c) in.q[c] = gq.p[c][o];  // written by the launch ahead
         return in;
     };
     unsigned rest = 0;  // rows whose pixel needs the general form

@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(256) k_prefilter(const __grid_constant__ FR p)
     for (int r = 0; r < 5; ++r) {
         const float *row = a.tmp + (int64_t)clampi(i + r - 2, 0, a.H - 1) * a.pitch;
 #pragma unroll
-        for (int c = 0; c < 5; ++c) s = fmaf(__ldg(a.w25 + r * 5 + c), __ldg(row + clampi(j + c - 2, 0, a.W - 1)), s);
+        for (int c = 0; c < 5; ++c) s = fmaf(__ldg(a.w25 + r * 5 + c), row[clampi(j + c - 2, 0, a.W - 1)], s);
     }
     st_store(static_cast<TS *>(a.out) + (int64_t)i * a.pitch + j, s);
 }
@@ -455,26 +455,27 @@ struct ReduceList {
 // Two horizontally adjacent outputs j = 2t, 2t+1 per thread: they share
 // input columns 4t-2 .. 4t+4 (7 loads per row instead of 10), loaded as
 // 8-byte pairs for FP32 storage away from the left and right borders.  Each
-// output is accumulated in the same order as the one-output form.
+// output is accumulated in the same order as the one-output form.  Ordinary
+// loads: the launch ahead may write the rows while this kernel is resident.
 template <typename TS>
 __device__ __forceinline__ void load7(const TS *row, int c0, int Ws, bool inside, float v[7])
 {
 #pragma unroll
-    for (int k = 0; k < 7; ++k) v[k] = ld_store(row + (inside ? c0 + k : clampi(c0 + k, 0, Ws - 1)));
+    for (int k = 0; k < 7; ++k) v[k] = to_f(row[inside ? c0 + k : clampi(c0 + k, 0, Ws - 1)]);
 }
 template <>
 __device__ __forceinline__ void load7<float>(const float *row, int c0, int Ws, bool inside, float v[7])
 {
     if (inside) {  // c0 even, row 8-byte aligned
-        const float2 a = __ldg(reinterpret_cast<const float2 *>(row + c0));
-        const float2 b = __ldg(reinterpret_cast<const float2 *>(row + c0 + 2));
-        const float2 c = __ldg(reinterpret_cast<const float2 *>(row + c0 + 4));
+        const float2 a = *reinterpret_cast<const float2 *>(row + c0);
+        const float2 b = *reinterpret_cast<const float2 *>(row + c0 + 2);
+        const float2 c = *reinterpret_cast<const float2 *>(row + c0 + 4);
         v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y; v[4] = c.x; v[5] = c.y;
-        v[6] = __ldg(row + c0 + 6);
+        v[6] = row[c0 + 6];
         return;
     }
 #pragma unroll
-    for (int k = 0; k < 7; ++k) v[k] = __ldg(row + clampi(c0 + k, 0, Ws - 1));
+    for (int k = 0; k < 7; ++k) v[k] = row[clampi(c0 + k, 0, Ws - 1)];
 }
 
 template <typename TS, typename FR>

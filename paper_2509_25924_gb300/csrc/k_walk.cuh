@@ -221,7 +221,7 @@ __device__ __forceinline__ void warp_compact(unsigned mask, const F &f)
 // products and pixels whose taps would be clamped go to the general sampler,
 // as do warps beyond the staged margin; those are gathered over the warp and
 // done together at the end.
-template <typename T, typename WS, bool COH, int MODE, bool EDGE>
+template <typename T, typename WS, int COH, int MODE, bool EDGE>
 __device__ __forceinline__ void walk_products(const IterArgs &a, int mode, const T *__restrict__ st1,
                                               const T *__restrict__ st2, int sx0, int sy0, int px0, int py0,
                                               float *prod, uint64_t *bars, int *err)
@@ -430,7 +430,7 @@ __device__ __forceinline__ void walk_vcolumn(float *col)
 
 // The guarded solve of G adjacent pixels and their store (gx a multiple of
 // G).  KEEP: the window sums go to a.s_out too (reverse mode).
-template <bool COH, bool KEEP, int G>
+template <int COH, bool KEEP, int G>
 __device__ __forceinline__ void walk_solve(const IterArgs &a, int mode, int gx, int gy, const float (&S)[5][G])
 {
     float2 V[G];
@@ -524,13 +524,15 @@ __device__ __forceinline__ void walk_fill_border(T *stage, int sx0, int sy0, int
 // One tile (the CTA's only one): the output pixels from (bx TX, row0 + by TY)
 // on, rows below row1 and the level's end.  TMA staging needs tensor maps
 // tm1, tm2 (box SP x SHB), or null, and NBAND mbarriers in shared memory.
-// CHAIN: the launch may have started before the one ahead of it ended; its
-// images are staged ahead of the wait for that launch if early.
-template <typename T, typename WS, bool COH, bool KEEP, bool CHAIN>
+// COH: how fields are read (FieldLoad).  CHAIN: the
+// launch may have started before the one ahead of it ended; its images are
+// staged ahead of the wait for that launch if early.
+template <typename T, typename WS, int COH, bool KEEP, bool CHAIN>
 __device__ __forceinline__ void walk_tile(const IterArgs &a, int mode, int bx, int by, int row0, int row1,
                                           float4 *smem_f4, const CUtensorMap *tm1, const CUtensorMap *tm2, int *err,
                                           uint64_t *tma_bars, bool early)
 {
+    static_assert(COH != LD_READ_ONLY || !CHAIN, "the launch ahead writes V0 while a chained one is resident");
     using SS = WalkStage<T, WS>;
     constexpr int TX = WS::TX, TY = WS::TY, R = WS::R, RW = WS::RW, P = WS::P, PLANE = WS::PLANE, NT = WS::NT;
     constexpr int SP = SS::SP, NV = SS::NV, VEC = SS::VEC, STG = SS::STG, SHT = SS::SHT, SHB = SS::SHB;

@@ -33,6 +33,16 @@ constexpr int kMaxFramesPerLaunch = kMaxPairsPerLaunch + 1;
 // it reads or writes what earlier work on the stream touches, and triggers
 // only after its own wait -- so whatever precedes the kernel before it is
 // complete even ahead of the wait.  Both are no-ops after a plain launch.
+//
+// Loads in such a kernel: it is resident while the kernel before it writes,
+// and __ldg (ld.global.nc) is for memory that nobody writes during the
+// kernel's lifetime, which the wait does not change.  What the kernel before
+// it may have written is read after the wait by ordinary loads (for V0 1 to 2 %
+// faster on single pairs than __ldcg, whose halo rows miss the L1);
+// __ldg serves what was complete before that kernel began: raw frames,
+// pre-filter weights, and the level images and earlier stages' fields once an
+// iteration has run.  (The first iteration after the pyramid starts from
+// V0 = 0, so its level images are read by the staging copies alone.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
