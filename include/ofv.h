@@ -401,10 +401,16 @@ ofv_status ofv_queue_selftest(int timeout_us, int *error_word);
  * 2x2 solve forms it (Eq. 2's normal equations are solved by Cramer's rule
  * with one reciprocal of the determinant): the hardware approximation
  * refined by one Newton-Raphson step.  x and y are device arrays of n
- * floats; for testing its error against 1/x. */
+ * floats; for testing its error against 1/x.
+ *
+ * ofv_debug_tma_levels(h, levels): *levels = number of pyramid levels whose
+ * iterations through ofv_compute and ofv_compute_sequence stage their image
+ * tiles by tensor copies, with the region mask as it is now (the others copy
+ * rows by cp.async: the same field, slower). */
 void ofv_debug_fail_alloc(int n);
 ofv_status ofv_debug_poison(ofv_handle *h, ofv_stream_t s);
 ofv_status ofv_debug_reciprocal(const float *x, float *y, int n, ofv_stream_t s);
+ofv_status ofv_debug_tma_levels(const ofv_handle *h, int *levels);
 
 /* ---- CUDA-graph replay (live loop) -------------------------------------
  * A live acquisition hands the estimator a new pair into the same device

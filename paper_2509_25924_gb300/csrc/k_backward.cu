@@ -855,8 +855,8 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
             a.s_out = w.Sst[sidx];
             a.s_plane = (size_t)h->Hs[l] * h->pitch[l];
             a.s_pitch = h->pitch[l];
-            const CUtensorMap *tm[2] = {&h->tmap[0][l], &h->tmap[1][l]};
-            const bool use = h->tma_ok[l] && h->tma_err_d;
+            const CUtensorMap *tm[2] = {&h->tmap[0][0][l], &h->tmap[0][1][l]};
+            const bool use = h->tma_ok[0][l] && h->tma_err_d;
             e = launch_iter_block(&a, 1, p.storage, stage_mode(sidx), s, use ? tm : nullptr, h->tma_err_d, 0, 0,
                                   tile_shape_of(p), sidx == 0 ? 1 : 2);
         } else {

@@ -93,18 +93,11 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
     // keep the window sums only for the reverse mode (uniform per launch)
     const bool var = a[0].inc || a[0].gauss || a[0].mask;
     const int kind = var ? ITER_VAR : a[0].s_out ? ITER_KEEP : overlap ? ITER_CHAIN : ITER_BOX;
-    if ((kind == ITER_VAR || kind == ITER_KEEP) && shape != 0) {
-        // these have the default tile shape only; tensor maps made for
-        // another shape's box would not match theirs
+    if (kind == ITER_VAR) shape = 0;  // its only shape, and that of its tensor maps' box
+    if (kind == ITER_KEEP && shape != 0) {
+        // tensor maps made for another shape's box would not match
         p.use_tma = 0;
         shape = 0;
-    }
-    if (kind == ITER_VAR && !a[0].gauss && !a[0].inc) {
-        // a mask set on a handle whose maps have the box-window kernels' box
-        int c0, r0, c1, r1;
-        block_stage_box(store, a[0].kr, &c0, &r0, 0, false);
-        block_stage_box(store, a[0].kr, &c1, &r1, 0, true);
-        if (c0 != c1 || r0 != r1) p.use_tma = 0;
     }
     if (kind != ITER_VAR && shape == 0 && npairs == 1 && walk_small_tiles(a[0].kr, a[0].W, p.row1 - row0)) shape = 1;
     switch (store) {

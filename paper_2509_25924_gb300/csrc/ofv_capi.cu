@@ -167,21 +167,20 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder_impl()
     return fn;
 }
 
-// Tensor maps of the level images for the block kernel's staged box (see
-// encode_block_map).  A level whose maps cannot be encoded keeps cp.async.
-void encode_tensor_maps(ofv_handle *h)
+// Tensor maps of the level images for the staged box of the iteration kernel
+// (see encode_block_map): set 0 of the handle's kernels, set 1 of a mask's
+// (the variants' kernels, default shape).  A level whose maps cannot be
+// encoded keeps cp.async.
+void encode_tensor_maps(ofv_handle *h, int set)
 {
-    int cols = 0, rows = 0;
-    const bool var = variant_of(h->p);
-    block_stage_box(h->p.storage, h->p.kernel_radius, &cols, &rows, tile_shape_of(h->p), var);
+    const bool var = set == 1 || variant_of(h->p);
+    const int shape = var ? 0 : tile_shape_of(h->p);
     for (int l = 0; l < h->L; ++l) {
-        h->tma_ok[l] = 0;
-        if (cols < 1) continue;
         bool ok = true;
         for (int f = 0; f < h->nslots && ok; ++f)
-            ok = encode_block_map(&h->tmap[f][l], h->lvl[f][l], h->Ws[l], h->Hs[l], h->pitch[l], h->p.storage,
-                                  h->p.kernel_radius, tile_shape_of(h->p), var);
-        h->tma_ok[l] = ok ? 1 : 0;
+            ok = encode_block_map(&h->tmap[set][f][l], h->lvl[f][l], h->Ws[l], h->Hs[l], h->pitch[l], h->p.storage,
+                                  h->p.kernel_radius, shape, var);
+        h->tma_ok[set][l] = ok ? 1 : 0;
     }
 }
 
@@ -324,11 +323,12 @@ ofv_status run_levels(ofv_handle *h, int np, const int *s1, const int *s2, float
             cudaError_t e = cudaSuccess;
             if (p.path == OFV_PATH_FUSED && block_supports(p.kernel_radius)) {
                 const CUtensorMap *tm[2 * kMaxBatch];
+                const int set = tma_set(h);
                 for (int k = 0; k < np; ++k) {
-                    tm[2 * k] = &h->tmap[s1[k]][l];
-                    tm[2 * k + 1] = &h->tmap[s2[k]][l];
+                    tm[2 * k] = &h->tmap[set][s1[k]][l];
+                    tm[2 * k + 1] = &h->tmap[set][s2[k]][l];
                 }
-                const bool use = h->tma_ok[l] && h->tma_err_d;
+                const bool use = h->tma_ok[set][l] && h->tma_err_d;
                 const bool first = l == h->L - 1 && t == 0;  // after the pyramid's launches
                 e = launch_iter_block(a, np, p.storage, mode, s, use ? tm : nullptr, h->tma_err_d, 0, 0,
                                       tile_shape_of(p), !overlap ? 0 : first ? 1 : 2);
@@ -690,7 +690,7 @@ ofv_status ofv_create(int H, int W, const ofv_params *p, ofv_handle **out)
         if (cudaHostAlloc(reinterpret_cast<void **>(&h->tma_err_h), sizeof(int), cudaHostAllocMapped) == cudaSuccess &&
             cudaHostGetDevicePointer(reinterpret_cast<void **>(&h->tma_err_d), h->tma_err_h, 0) == cudaSuccess) {
             *h->tma_err_h = 0;
-            encode_tensor_maps(h);
+            encode_tensor_maps(h, 0);
         } else {
             cudaGetLastError();
             if (h->tma_err_h) cudaFreeHost(h->tma_err_h);
@@ -763,6 +763,15 @@ ofv_status ofv_debug_poison(ofv_handle *h, ofv_stream_t s)
     return e == cudaSuccess ? OFV_OK : cuda_fail(e, "poisoning the workspace");
 }
 
+ofv_status ofv_debug_tma_levels(const ofv_handle *h, int *levels)
+{
+    if (!h || !levels) return fail(OFV_ERR_INVALID_ARG, "handle or levels is NULL");
+    *levels = 0;
+    if (h->tma_err_d)
+        for (int l = 0; l < h->L; ++l) *levels += h->tma_ok[tma_set(h)][l];
+    return OFV_OK;
+}
+
 ofv_status ofv_set_mask(ofv_handle *h, const uint8_t *mask, ofv_stream_t s)
 {
     if (!h) return fail(OFV_ERR_INVALID_ARG, "handle is NULL");
@@ -784,6 +793,7 @@ ofv_status ofv_set_mask(ofv_handle *h, const uint8_t *mask, ofv_stream_t s)
             return fail(OFV_ERR_ALLOC, "cudaMalloc of %zu mask bytes failed", total);
         }
         for (int l = 0; l < h->L; ++l) h->mask_lvl[l] = static_cast<uint8_t *>(h->mask_arena) + off[l];
+        if (h->tma_err_d) encode_tensor_maps(h, 1);
     }
     cudaError_t e = launch_mask_levels(mask, h->W, h->mask_lvl, h->Hs, h->Ws, h->L, (cudaStream_t)s);
     if (e != cudaSuccess) return cuda_fail(e, "mask level launch");

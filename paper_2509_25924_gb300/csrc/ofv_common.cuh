@@ -124,9 +124,11 @@ inline void set_iter_variant(IterArgs &a, int kr, int window_gauss, float sigma,
 cudaError_t launch_iter_fused(const IterArgs &a, int store, int mode, cudaStream_t s);
 // Block-tiled kernel (KR 1..10): npairs pairs of equal level size in one launch.
 // tm (optional): 2 * npairs tensor maps (frame 1 and frame 2 of pair k at
-// 2k, 2k+1) of the level images with the box of block_stage_box; tiles whose
-// staged box lies inside the image are then loaded by TMA.  err (optional):
-// device-visible word set to 1 if a TMA wait expires.
+// 2k, 2k+1) of the level images with the box of block_stage_box for the
+// kernel that runs (the variants' with a mask too); tiles are then loaded by
+// TMA, those of the variants' kernels only where the staged box lies inside
+// the image.  err (optional): device-visible word set to 1 if a TMA wait
+// expires.
 bool block_supports(int kr);
 // The forward solve's reciprocal of x[0..n-1] into y (device arrays), for tests.
 cudaError_t launch_recip(const float *x, float *y, int n, cudaStream_t s);
@@ -142,7 +144,7 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
                               int shape = 0, int overlap = 0);
 // TMA box of the iteration kernels' staging (columns, rows of one band) for
 // this storage, radius and tile shape; var: of the estimator variants'
-// kernels (Gaussian window, increment form).
+// kernels (Gaussian window, increment form, region mask).
 void block_stage_box(int store, int kr, int *cols, int *rows, int shape = 0, bool var = false);
 
 struct PlainBufs {

@@ -89,11 +89,13 @@ struct ofv_handle {
     // every strip's pyramids and fields
     void *strip_arena;
     size_t strip_bytes;
-    // TMA tensor maps of every (slot, level) image for the block kernel's
-    // staged box, and the word a kernel sets when a TMA wait expires
-    // (page-locked host memory mapped into the device)
-    CUtensorMap tmap[ofv::kMaxSlots][ofv::kMaxLevels];
-    int tma_ok[ofv::kMaxLevels];
+    // TMA tensor maps of every (slot, level) image for the iteration kernel's
+    // staged box -- [0] of the handle's kernels, [1] of the kernels that a
+    // region mask takes (encoded with the first mask; see tma_set) -- and the
+    // word a kernel sets when a TMA wait expires (page-locked host memory
+    // mapped into the device)
+    CUtensorMap tmap[2][ofv::kMaxSlots][ofv::kMaxLevels];
+    int tma_ok[2][ofv::kMaxLevels];
     int *tma_err_h, *tma_err_d;
     // host-memory sequence pipeline: copy streams, ring events, device ring
     cudaStream_t hs_stream[2];            // [0] host-to-device, [1] device-to-host
@@ -135,6 +137,9 @@ bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch,
                       bool var = false);
 // The estimator variants whose kernels a handle runs throughout.
 inline bool variant_of(const ofv_params &p) { return p.window == OFV_WINDOW_GAUSS || p.increment_form; }
+// Which tensor maps an iteration of this handle takes now: the variants'
+// kernels, which a mask runs, have a staged box of their own.
+inline int tma_set(const ofv_handle *h) { return h->mask_on && !variant_of(h->p) ? 1 : 0; }
 // Tile shape of the block kernel that params select: 0 (default) or 1 (the
 // alternative edge), -1 when tile_edge is not one of the radius's edges on
 // the fused block path.  The Gaussian window and the increment form run the

@@ -320,6 +320,48 @@ def test_masked_sequence_and_clearing_the_mask():
         ofv.ofv_destroy(h)
 
 
+@pytest.mark.parametrize("kr,storage,edge", [(1, ofv.OFV_STORE_F32, 0), (3, ofv.OFV_STORE_F32, 0),
+                                             (4, ofv.OFV_STORE_F32, 32), (4, ofv.OFV_STORE_F16, 0),
+                                             (5, ofv.OFV_STORE_BF16, 0), (6, ofv.OFV_STORE_F32, 32),
+                                             (10, ofv.OFV_STORE_F32, 0)])
+def test_masked_launches_stage_by_tensor_copies_as_unmasked_ones_do(kr, storage, edge):
+    """The kernels a mask runs have a staged box of their own: with tensor maps
+    of the box window's kernels they would copy their tiles row by row."""
+    H, W = 230, 300
+    I1, I2 = (I.astype(np.float32) for I in synth.smooth_pair(H, W, (1.3, -0.7), seed=12))
+    m = _disk_and_band_mask(H, W)
+    kw = dict(levels_psl=1, kernel_radius=kr, iterations=2)
+    h = ofv.ofv_create(H, W, ofv.ofv_default_params(input=ofv.OFV_IN_F32, storage=storage, tile_edge=edge, **kw))
+    try:
+        assert ofv.ofv_debug_tma_levels(h) == 2
+        t1, t2 = torch.from_numpy(I1).to(DEV), torch.from_numpy(I2).to(DEV)
+        u0 = torch.empty((H, W), device=DEV); v0 = torch.empty_like(u0)
+        ofv.ofv_compute(h, t1, t2, u0, v0)
+        ofv.ofv_set_mask(h, torch.from_numpy(m).to(DEV))
+        assert ofv.ofv_debug_tma_levels(h) == 2
+        u = torch.empty_like(u0); v = torch.empty_like(u0)
+        ofv.ofv_compute(h, t1, t2, u, v)
+        ofv.ofv_set_mask(h, None)
+        assert ofv.ofv_debug_tma_levels(h) == 2
+        u1 = torch.empty_like(u0); v1 = torch.empty_like(u0)
+        ofv.ofv_compute(h, t1, t2, u1, v1)
+        torch.cuda.synchronize()
+        assert torch.equal(u1, u0) and torch.equal(v1, v0)
+    finally:
+        ofv.ofv_destroy(h)
+    ou, ov, nd, _ = oracle.flow(I1.astype(np.float64), I2.astype(np.float64),
+                                oracle.Params(psl=1, kr=kr, it=2, mask=m), diagnostics=True)
+    u, v = u.cpu().numpy(), v.cpu().numpy()
+    assert np.array_equal(np.isnan(u), m == 0)
+    sel = m != 0
+    # a 3x3 window leaves more pixels nearly singular; 16-bit levels by the RMS rule
+    if storage == ofv.OFV_STORE_F32:
+        _compare(u[sel], v[sel], ou[sel], ov[sel], nd[sel], f"mask kr{kr}", max_masked=0.05 if kr == 1 else 0.01)
+    else:
+        d = np.hypot(u[sel] - ou[sel], v[sel] - ov[sel])[nd[sel] >= 1e-3]
+        assert np.sqrt(np.mean(d ** 2)) <= 1e-2
+
+
 def test_graph_replay_runs_the_variants_and_the_mask_like_compute(rankine):
     """A CUDA graph recorded with the Gaussian window, the increment form and
     a region mask replays bitwise the field of ofv_compute."""
