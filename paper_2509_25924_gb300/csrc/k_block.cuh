@@ -548,7 +548,7 @@ __device__ __forceinline__ void products_tile_interior(const IterArgs &a, const 
 // one; a step writes only its own block's outputs, whose values are already
 // in registers, so the line can be overwritten in place.
 template <int KR, int TS, bool TAIL>
-__device__ __forceinline__ void window_step(float *line, int stride, int b0, float (&cur)[2 * KR + 1])
+__host__ __device__ __forceinline__ void window_step(float *line, int stride, int b0, float (&cur)[2 * KR + 1])
 {
     constexpr int WIN = 2 * KR + 1, N = TS + 2 * KR;
     float nxt[WIN];
@@ -568,7 +568,7 @@ __device__ __forceinline__ void window_step(float *line, int stride, int b0, flo
 }
 
 template <int KR, int TS>
-__device__ __forceinline__ void window_sums_inplace(float *line, int stride)
+__host__ __device__ __forceinline__ void window_sums_inplace(float *line, int stride)
 {
     constexpr int WIN = 2 * KR + 1, N = TS + 2 * KR;
     constexpr int NFULL = (N - WIN) / WIN;  // steps whose next block lies wholly inside the line

@@ -57,8 +57,10 @@ template <int R_, int SHAPE_> struct WalkShape {
     static constexpr int NSEG = R <= 4 ? (TY == 40 ? 6 : 4) : SHAPE == 1 ? 6 : R == 5 ? 8 : 12;  // segments of a column
     static constexpr int NROW = (RH + NSEG - 1) / NSEG;      // rows a thread walks
     static constexpr int NT = COLS ? 32 * NW * NSEG : R == 5 ? 480 : 1024;
-    // resident CTAs per SM
-    static constexpr int MINB = R <= 4 ? (TY == 40 ? 2 : 3) : SHAPE == 0 ? (R == 5 ? 2 : 1) : R <= 8 ? 2 : 1;
+    // resident CTAs per SM (the launch bound keeps radii 9 and 10 of the smaller
+    // shape at 80 registers: with 85 only one of the two CTAs fits, 32 fields of
+    // 1 Mp at R 10 4.55 instead of 3.08 ms)
+    static constexpr int MINB = R <= 4 ? (TY == 40 ? 2 : 3) : SHAPE == 0 && R > 5 ? 1 : 2;
     static constexpr bool ALL = COLS && RW % 32 == 0 && RH == NSEG * NROW;  // every thread stores NROW pixels
     // row pitch of the product planes: an odd multiple of 4, so that octets
     // of lanes on two rows, eight columns apart, read distinct banks in phase 3
@@ -366,15 +368,19 @@ __device__ __forceinline__ void walk_products(const IterArgs &a, int mode, const
     });
 }
 
-__device__ __forceinline__ float add_v(float a, float b) { return a + b; }
+__host__ __device__ __forceinline__ float add_v(float a, float b) { return a + b; }
 __device__ __forceinline__ float2 add_v(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
 // Window sums of G consecutive outputs from the G + 2R values load(0) ..
 // load(G + 2R - 1), in registers: blocks of up to 2R+1 outputs share a core
 // of values, which running sums extend downwards in index (into o[]) and
-// upwards (pre).  Additions only; each value is loaded once.
+// upwards (pre).  Additions only; each value is loaded once.  A core of four
+// values or more is summed in halves: in one chain a sum of 21 values rounds 20
+// times in a row, which left the fields of R 8 .. 10 up to 4 % further off the
+// 64-bit ones than the block decomposition (R 10: 1.06e-7 relative against
+// 1.03e-7; in halves 0.98e-7), at the same speed.
 template <int R, int G, typename V, typename Load>
-__device__ __forceinline__ void window_group(const Load &load, V (&o)[G])
+__host__ __device__ __forceinline__ void window_group(const Load &load, V (&o)[G])
 {
     constexpr int WIN = 2 * R + 1;
     V v[G + 2 * R];
@@ -386,9 +392,16 @@ __device__ __forceinline__ void window_group(const Load &load, V (&o)[G])
             if (r >= old) v[r] = load(r);
             return v[r];
         };
+        const int n = WIN + 1 - m, half = n >= 4 ? (n + 1) / 2 : n;  // values of the core, of its first part
         V s = val(b + m - 1);
 #pragma unroll
-        for (int r = b + m; r <= b + 2 * R; ++r) s = add_v(s, val(r));
+        for (int r = 1; r < half; ++r) s = add_v(s, val(b + m - 1 + r));
+        if (n > half) {
+            V t = val(b + m - 1 + half);
+#pragma unroll
+            for (int r = half + 1; r < n; ++r) t = add_v(t, val(b + m - 1 + r));
+            s = add_v(s, t);
+        }
         o[b + m - 1] = s;
 #pragma unroll
         for (int k = m - 2; k >= 0; --k) {

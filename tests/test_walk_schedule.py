@@ -15,14 +15,25 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_2509_25924_gb300", "csrc")
 
 
-def test_walk_items_taps_and_bands(tmp_path):
+def _run_check(tmp_path, name):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not found")
-    exe = tmp_path / "walk_schedule_check"
-    subprocess.check_call([nvcc, "-std=c++17", "-I", CSRC, "-gencode", "arch=compute_103a,code=sm_103a",
-                           os.path.join(HERE, "walk_schedule_check.cu"), "-o", str(exe)])
+    exe = tmp_path / name
+    subprocess.check_call([nvcc, "-std=c++17", "--expt-relaxed-constexpr", "-I", CSRC, "-gencode",
+                           "arch=compute_103a,code=sm_103a", os.path.join(HERE, name + ".cu"), "-o", str(exe)])
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
-    lines = out.stdout.splitlines()
+    return out.stdout.splitlines()
+
+
+def test_walk_items_taps_and_bands(tmp_path):
+    lines = _run_check(tmp_path, "walk_schedule_check")
     assert len(lines) == 3 * 20 + 1 and lines[-1] == "0 failing cases"
+
+
+def test_window_sums_round_no_worse_than_the_block_form(tmp_path):
+    # a sum of (2R+1)^2 products keeps the error of the block decomposition,
+    # although its groups of eight outputs share a core of values
+    lines = _run_check(tmp_path, "window_sum_check")
+    assert len(lines) == 11 and lines[-1] == "0 failing radii"
