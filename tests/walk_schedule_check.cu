@@ -9,7 +9,9 @@
 //     of the region, and the output groups cover the tile once, with loads
 //     inside a plane's row and octets of lanes on distinct banks;
 //   * the staged box is one TMA can copy and the tile fits its share of
-//     shared memory.
+//     shared memory;
+//   * no further segment of a column that would shorten the walks fits the
+//     threads.
 // Prints one line per case and "FAIL" on any violation.
 #include <cstdio>
 #include <cstring>
@@ -94,6 +96,7 @@ static int check(const char *tname)
     if (SS::band_row(SS::NBAND - 1) + SS::SHB != SS::SHT || SS::STG < SS::SHT * SP) ++bad;
     const size_t smem = walk_smem_bytes<T, WS>();
     if (WS::MINB * (smem + 1024 + 32) > 228 * 1024 || smem > 227 * 1024 - 512) ++bad;
+    if (!WS::COLS && (WS::NSEG + 1) * RW <= WS::NT && (RH + WS::NSEG) / (WS::NSEG + 1) < NROW) ++bad;
     if (WS::TX != walk_tile_w(R, SHAPE) || WS::TY != walk_tile_h(R, SHAPE)) ++bad;
     printf("%s KR %2d tile %2dx%2d NT %4d rows %d SP %d P %d smem %zu bad %d%s\n", tname, R, WS::TX, WS::TY, WS::NT,
            NROW, SP, P, smem, bad, bad ? " FAIL" : "");
