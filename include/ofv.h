@@ -265,9 +265,9 @@ ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2, const flo
  * raise the rate further (Conclusions).  ofv_compute_strips computes one
  * field as nstrips horizontal strips, each with a workspace of its own (here
  * all on the handle's device, one strip after another on stream s): at
- * every level a strip owns whole tile rows of the block kernel's tile grid
- * and computes the rows of its pyramids it reads (own rows plus a redundant
- * halo, from the input rows around them), so images need no exchange; after
+ * every level a strip owns whole rows of tile_edge pixels and computes the
+ * rows of its pyramids that these depend on (own rows plus a redundant halo,
+ * from the input rows around them), so images need no exchange; after
  * every Gauss-Newton iteration it copies from their owners the rows of the
  * new field its next iteration reads (the window halo, or the coarse rows
  * the next level's up-sampling reads).  The field equals ofv_compute's
@@ -277,9 +277,10 @@ ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2, const flo
  * pyramids and two fields, grown on demand and owned by the handle; I1, I2,
  * u, v as for ofv_compute. */
 typedef struct {
-    int own_row0, own_row1;       /* rows of the level the strip outputs (whole tile rows) */
+    int own_row0, own_row1;       /* rows of the level the strip outputs (whole rows of tile_edge px) */
     int img_row0, img_row1;       /* rows of the level's images it computes (own rows and the halo) */
-    int fld_row0, fld_row1;       /* rows of the level's field its iterations read */
+    int fld_row0, fld_row1;       /* rows of the level's field its outputs depend on (a tile that runs past
+                                     the own rows reads on, without effect: buffers have the level's size) */
     int up_row0, up_row1;         /* rows of the next coarser level's field read when up-sampling to this level */
     int ingest_row0, ingest_row1; /* level 0: input rows it ingests (0, 0 at other levels) */
 } ofv_strip_rows;

@@ -3,9 +3,16 @@
 // several GPUs (the paper names 2 or 3 GPUs as the way to raise the rate
 // further, Conclusions), here run strip after strip on one device.
 //
-// At every level the strips own whole tile rows of the block kernel's tile
-// grid (so each output pixel is computed by the same tile, with the same
-// window-sum order, as in the single-field computation).  A strip builds the
+// At every level the strips own whole rows of tile_edge pixels, which start
+// at multiples of the window sums' units of eight rows, so each output pixel
+// has the same window-sum order as in the single-field computation.  The tiles
+// start at a strip's first row and are 24 to 64 rows high, so the last row of
+// them may run past the rows owned, by up to 32; what it reads there (image
+// rows and V0 that the strip did not compute) goes into products that no owned
+// output sums, and its outputs there are not stored.  The buffers therefore
+// have the level's full size; ofv_strip_plan lists the rows that the owned
+// outputs depend on.  (Bounding the tiles at those rows instead cost the
+// iteration kernel 0.2 to 1.4 % on fields without strips.)  A strip builds the
 // rows of its pyramid it reads -- its own rows plus a redundant image halo
 // wide enough for the staged tiles, the window and warps up to max_disp --
 // from an input view of the rows below and above it, so images need no
@@ -79,9 +86,10 @@ ofv_status plan_strip(int H, int W, const ofv_params &p, int nstrips, int max_di
         }
         // products of the tiles' window halo read V0 there
         o->fld[l] = clip(Range{o->own[l].a - KR, o->own[l].b + KR}, Hl);
-        // images: the staged box of a tile reaches KR + REACH + 4 rows past
-        // the tile, and the three staging bands up to 2 more; warps beyond the
-        // staged margin read up to |V|/2 + 2 rows away (V of the level)
+        // images: products up to KR rows away sample up to REACH + 2 rows from
+        // their pixel within the staged margin (8 allows for the variants'
+        // staging bands); warps beyond it read up to |V|/2 + 2 rows away (V of
+        // the level)
         const int warp = (max_disp + (1 << (l + 1)) - 1) / (1 << (l + 1)) + 2;
         const int margin = KR + kBlockReach + 8 + warp;
         need[l] = clip(Range{o->own[l].a - margin, o->own[l].b + margin}, Hl);
@@ -155,7 +163,7 @@ extern "C" ofv_status ofv_strip_plan(int H, int W, const ofv_params *params, int
 namespace {
 
 // Workspace of one strip: its pyramids of both frames and two ping-pong fields
-// (full-size buffers, of which it computes only its rows).
+// (full-size buffers, of which it computes only its rows; see the top).
 struct StripBufs {
     void *lvl[2][kMaxLevels];
     float2 *fld[2];
