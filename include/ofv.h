@@ -116,8 +116,9 @@ typedef struct {
                            the two per batch signature (ofv_batch_tuning reports it); nonzero fixes it.
                            The edge is the unit of rows of a strip and selects the larger or the smaller
                            tiles; the order of a pixel's window sums follows its position in the image,
-                           so all tiles give the same field bitwise.  The estimator variants (Gaussian
-                           window, increment form, region mask) and the reverse mode run the default. */
+                           so all tiles give the same field bitwise (KR 1 and 2 have one tile for both).
+                           The estimator variants (Gaussian window, increment form, region mask) run the
+                           default, the reverse mode from KR 5 on too. */
 } ofv_params;
 
 typedef struct ofv_handle ofv_handle;

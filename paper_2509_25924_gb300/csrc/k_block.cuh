@@ -74,7 +74,9 @@ __host__ __device__ constexpr int block_tile_edge(int kr, int v)
 }
 
 // Output tile of the box-window kernels (k_walk.cuh), which give the same
-// field whatever their tiles: the default and the smaller alternative.
+// field whatever their tiles: the default and, for radii above 2, a smaller
+// alternative.
+__host__ __device__ constexpr bool walk_has_alt(int kr) { return kr > 2; }
 __host__ __device__ constexpr int walk_tile_w(int kr, int v)
 {
     return kr <= 4 ? 56 : v == 0 ? (kr == 5 ? 48 : 64) : kr <= 8 ? 48 : 40;

@@ -175,17 +175,20 @@ cudaError_t run_block(const BlockParams &p, dim3 grid, int dev, cudaStream_t s)
 // KS = kr + 16 shape for the radii and shapes instantiated here: every
 // radius with its default shape; the alternative shapes without the
 // estimator variants (keeping the window sums, of radii 3 and 4, whose small
-// levels take them).  0 when not instantiated.
+// levels take them).  Box windows of radii 1 and 2, whose two shapes are one
+// tile, run the default for both.  0 when not instantiated.
 template <int KIND>
 constexpr bool has_alt(int kr)
 {
-    return KIND == ITER_BOX || KIND == ITER_CHAIN || (KIND == ITER_KEEP && (kr == 3 || kr == 4));
+    return walk_has_alt(kr) &&
+           (KIND == ITER_BOX || KIND == ITER_CHAIN || (KIND == ITER_KEEP && (kr == 3 || kr == 4)));
 }
 template <int KIND>
 constexpr int ks_of(int kr, int shape)
 {
-    return kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1 || (shape != 0 && !has_alt<KIND>(kr)) ? 0
-                                                                                                 : kr + 16 * shape;
+    if (kr < 1 || kr > kBlockMaxKR || shape < 0 || shape > 1) return 0;
+    if (KIND != ITER_VAR && !walk_has_alt(kr)) shape = 0;
+    return shape != 0 && !has_alt<KIND>(kr) ? 0 : kr + 16 * shape;
 }
 
 #define OFV_KS_CASES(X)                                                                                    \

@@ -94,8 +94,9 @@ cudaError_t launch_iter_block(const IterArgs *a, int npairs, int store, int mode
     const bool var = a[0].inc || a[0].gauss || a[0].mask;
     const int kind = var ? ITER_VAR : a[0].s_out ? ITER_KEEP : overlap ? ITER_CHAIN : ITER_BOX;
     if (kind == ITER_VAR) shape = 0;  // its only shape, and that of its tensor maps' box
-    if (kind == ITER_KEEP && shape != 0) {
-        // tensor maps made for another shape's box would not match
+    if (kind == ITER_KEEP && shape != 0 && a[0].kr > 4) {
+        // the default shape only, whose box tensor maps made for the other one
+        // would not match; up to radius 4 the shapes share the box
         p.use_tma = 0;
         shape = 0;
     }

@@ -111,9 +111,10 @@ ofv_status batched_impl(ofv_handle *h, int n, const ofv_pair *pairs, ofv_stream_
     const int sb = store_bytes(p.storage);
     const bool var = p.window == OFV_WINDOW_GAUSS || p.increment_form;
     // tile shapes the tuner may pick: the one tile_edge names, else both
-    // (the variant kernels have the default shape only)
+    // (the variant kernels have the default shape only, and the tiles of radii
+    // 1 and 2 one shape)
     std::vector<int> shapes;
-    if (p.tile_edge != 0 || var)
+    if (p.tile_edge != 0 || var || !walk_has_alt(KR))
         shapes.push_back(std::max(tile_shape_of(p), 0));
     else
         shapes = {0, 1};

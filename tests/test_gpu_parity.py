@@ -673,6 +673,29 @@ def test_batched_other_radii_and_storage(kr, storage):
         ofv.ofv_destroy(h)
 
 
+@pytest.mark.parametrize("kr", [1, 2])
+def test_batch_of_a_radius_with_one_tile_has_one_shape_to_tune(kr):
+    """Both tile shapes of radii 1 and 2 are one tile: the tuner has the default
+    only, a fixed edge of 32 is kept, and the fields are the same."""
+    sizes = [(200, 232), (130, 320), (96, 130)]
+    data = _uneven_pairs(sizes, seed0=500 + kr)
+    fields = []
+    for edge in (0, 32):
+        h = ofv.ofv_create(64, 64, ofv.ofv_default_params(levels_psl=1, kernel_radius=kr, iterations=2, tile_edge=edge))
+        try:
+            bufs = [(torch.from_numpy(I1).to(DEV), torch.from_numpy(I2).to(DEV),
+                     torch.full((H, W), float("nan"), device=DEV), torch.full((H, W), float("nan"), device=DEV))
+                    for (I1, I2), (H, W) in zip(data, sizes)]
+            ofv.ofv_compute_batched(h, bufs)
+            torch.cuda.synchronize()
+            assert ofv.ofv_batch_tuning(h)["tile_edge"] == (edge or 48)
+            fields.append([b[2:] for b in bufs])
+        finally:
+            ofv.ofv_destroy(h)
+    for (u0, v0), (u1, v1) in zip(*fields):
+        assert torch.equal(u0, u1) and torch.equal(v0, v1) and torch.isfinite(u0).all()
+
+
 def test_batched_graph_replays_the_batch_and_keeps_its_own_workspace():
     """ofv_graph_create_batched records the batch; a replay gives bitwise the
     eager batch's fields, follows new frames written into the same buffers,

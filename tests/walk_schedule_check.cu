@@ -10,6 +10,7 @@
 //     inside a plane's row and octets of lanes on distinct banks;
 //   * the staged box is one TMA can copy and the tile fits its share of
 //     shared memory;
+//   * the smaller shape is another tile where walk_has_alt says so;
 //   * no further segment of a column that would shorten the walks fits the
 //     threads.
 // Prints one line per case and "FAIL" on any violation.
@@ -96,6 +97,11 @@ static int check(const char *tname)
     if (SS::band_row(SS::NBAND - 1) + SS::SHB != SS::SHT || SS::STG < SS::SHT * SP) ++bad;
     const size_t smem = walk_smem_bytes<T, WS>();
     if (WS::MINB * (smem + 1024 + 32) > 228 * 1024 || smem > 227 * 1024 - 512) ++bad;
+    if (SHAPE == 1) {
+        using W0 = WalkShape<R, 0>;
+        const bool same = W0::TX == WS::TX && W0::TY == WS::TY && W0::NT == WS::NT;
+        if (same == walk_has_alt(R)) ++bad;
+    }
     if (!WS::COLS && (WS::NSEG + 1) * RW <= WS::NT && (RH + WS::NSEG) / (WS::NSEG + 1) < NROW) ++bad;
     if (WS::TX != walk_tile_w(R, SHAPE) || WS::TY != walk_tile_h(R, SHAPE)) ++bad;
     printf("%s KR %2d tile %2dx%2d NT %4d rows %d SP %d P %d smem %zu bad %d%s\n", tname, R, WS::TX, WS::TY, WS::NT,
