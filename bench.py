@@ -181,14 +181,19 @@ def run_reference(args, ws, rank):
 # ---------------------------------------------------------------------------
 # our arm
 # ---------------------------------------------------------------------------
+KERNEL_SOURCES = ("k_walk.cuh", "k_block.cuh", "k_block_inst.cuh", "iter_math.cuh", "ofv_common.cuh")
+
+
 def kernel_source_hash():
     """Hash of the iteration kernel's sources with comments and blank lines
-    removed: it changes when the code changes, not when a comment does."""
+    removed: it changes when the code changes or a source is missing, not when
+    a comment does."""
     import re
     h = hashlib.sha256()
-    for f in ("k_walk.cuh", "k_block.cuh", "k_block_inst.cuh", "iter_math.cuh", "ofv_common.cuh"):
+    for f in KERNEL_SOURCES:
         path = os.path.join(ROOT, "paper_2509_25924_gb300", "csrc", f)
         if not os.path.exists(path):
+            h.update(f"{f} is missing".encode())
             continue
         with open(path) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)

@@ -33,5 +33,19 @@ def test_kernel_hash_follows_code_not_comments(tmp_path, monkeypatch):
     assert bench.kernel_source_hash() != h0
 
 
+def test_kernel_hash_covers_every_source_it_names(tmp_path, monkeypatch):
+    """A source that is renamed must not leave the record's key in silence."""
+    csrc = os.path.join(ROOT, "paper_2509_25924_gb300", "csrc")
+    assert all(os.path.exists(os.path.join(csrc, f)) for f in bench.KERNEL_SOURCES)
+    d = _copy_sources(tmp_path)
+    shutil.copy(os.path.join(csrc, "k_walk.cuh"), d / "k_walk.cuh")
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    seen = {bench.kernel_source_hash()}
+    for f in bench.KERNEL_SOURCES:
+        os.rename(d / f, d / ("x_" + f))
+        seen.add(bench.kernel_source_hash())
+    assert len(seen) == 1 + len(bench.KERNEL_SOURCES)
+
+
 def test_whole_job_rate_counts_every_rank():
     assert bench.whole_job_rate(1000, 4, 2.0) == 2000.0
