@@ -751,7 +751,7 @@ def live_loop(ofv, torch, synth, dev, stream, n_pairs=2000, ring=8, lanes=1, pap
 def batched_uneven(ofv, torch, synth, dev, stream, n_pairs=64, reps=5):
     """64 pairs with sizes drawn (seed 5) from {256^2, 512^2, 768x1024,
     1024^2}, turbulence displacement: one ofv_compute_batched call (one
-    persistent launch for all iterations) vs one ofv_compute per pair.  Each
+    launch for all iterations) vs one ofv_compute per pair.  Each
     pair has its own device buffers; pairs of one size class share content."""
     classes = [(256, 256), (512, 512), (768, 1024), (1024, 1024)]
     rng = np.random.default_rng(5)

@@ -13,10 +13,11 @@
 //            taps (atomics) and differentiate with respect to the position,
 //            which gives the gradient of V0 (clamped taps: zero slope beyond
 //            the border);
-//   then the up-sampling (scatter to the coarse field), the pyramid
-//   reductions (scatter) and the pre-filter (transpose and weight
-//   gradient).  Float atomics make the summation order, and so the last bits,
-//   vary from run to run.
+//   then the transposes of the up-sampling, the pyramid reductions and the
+//   pre-filter (with its weight gradient), each gathered by the pixel it
+//   writes.  Float atomics, of the samples and of the weight gradient's sum over
+//   the CTAs, make the summation order, and so the last bits, vary from run to
+//   run.
 #include <cstring>
 
 #include "iter_math.cuh"
@@ -903,12 +904,8 @@ extern "C" ofv_status ofv_backward(ofv_handle *h, const void *I1, const void *I2
         BW_TRY(cudaMemsetAsync(gw25, 0, 25 * sizeof(float), s), "ofv_backward: memset");
     }
     if (p.norm_radius > 0) {
-        // the ten level-0 planes of A and B are free now: dense H x W scratch
-        float *t[10];
-        for (int c = 0; c < 5; ++c) {
-            t[c] = w.A.p[c];
-            t[5 + c] = w.B.p[c];
-        }
+        // the level-0 planes of A are free now: dense H x W scratch
+        float *const t[4] = {w.A.p[0], w.A.p[1], w.A.p[2], w.A.p[3]};
         BW_TRY(bw_input_norm(w.gP1[0], h->pitch[0], h->H, h->W, I1, p.input, scale, p.norm_radius, p.norm_eps,
                              h->w25, p.prefilter, gI1, gw, t, s),
                "ofv_backward: normalization adjoint");

@@ -250,7 +250,7 @@ int queue_occupancy_kr()
     return n;
 }
 
-// The variants' persistent kernel has its own thread count: KS | 32 (see
+// The variants' batched kernel has its own thread count: KS | 32 (see
 // BlockShape).
 #define QKS(K) (KIND == ITER_VAR ? ((K) | 32) : (K))
 

@@ -30,12 +30,9 @@ struct IngestList {
     __device__ __forceinline__ const IngestArgs &get(int k) const { return f[k]; }
 };
 
-// Scaled intensity I = raw * scale (scale = 1/(2^bits - 1), or 1 for FP32
-// input), then, for NR > 0, (I - mu) / sqrt(var + eps_n^2) with mu and var
-// taken over the in-image part of the (2NR+1)^2 box.  Writes level 0 in the
-// storage type, or FP32 scratch when a pre-filter follows.  With NR > 0 it
-// serves only NR > 16 (k_ingest_norm below covers 1 .. 16, with the mean
-// from separable sums: the two agree to FP32 rounding).
+// Without normalization: scaled intensity I = raw * scale (scale =
+// 1/(2^bits - 1), or 1 for FP32 input), to level 0 in the storage type, or to
+// FP32 scratch when a pre-filter follows.
 template <typename TI, typename TS, typename FR>
 __global__ void __launch_bounds__(256) k_ingest(const __grid_constant__ FR p)
 {
@@ -44,36 +41,18 @@ __global__ void __launch_bounds__(256) k_ingest(const __grid_constant__ FR p)
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= a.H || j >= a.W) return;
-    const TI *raw = static_cast<const TI *>(a.raw);
-    const float sc = p.scale;
-    float val = ld_in(raw + (int64_t)i * a.W + j) * sc;
-    if (a.nr > 0) {
-        const int i0 = max(i - a.nr, 0), i1 = min(i + a.nr, a.H - 1);
-        const int j0 = max(j - a.nr, 0), j1 = min(j + a.nr, a.W - 1);
-        const float inv_n = 1.0f / (float)((i1 - i0 + 1) * (j1 - j0 + 1));
-        float s = 0.f;
-        for (int ii = i0; ii <= i1; ++ii)
-            for (int jj = j0; jj <= j1; ++jj) s += ld_in(raw + (int64_t)ii * a.W + jj) * sc;
-        const float mu = s * inv_n;
-        float q = 0.f;
-        for (int ii = i0; ii <= i1; ++ii)
-            for (int jj = j0; jj <= j1; ++jj) {
-                const float d = ld_in(raw + (int64_t)ii * a.W + jj) * sc - mu;
-                q = fmaf(d, d, q);
-            }
-        const float var = q * inv_n;
-        val = (val - mu) * rsqrtf(var + a.eps_n * a.eps_n);
-    }
+    const float val = ld_in(static_cast<const TI *>(a.raw) + (int64_t)i * a.W + j) * p.scale;
     if (a.prefilter)
         a.tmp[(int64_t)i * a.pitch + j] = val;
     else
         st_store(static_cast<TS *>(a.out) + (int64_t)i * a.pitch + j, val);
 }
 
-// The same for FP32 frames with the boxes in shared memory: a CTA of 32 x 8 threads stages
-// a 32 x 32 block (four rows per thread) and the NR halo (scaled values,
-// zero outside the image, so the boxes are truncated there).  The mean comes from separable sums:
-// row sums over 2NR+1 columns for every staged row, then 2NR+1 of them down
+// Local normalization, NR 1 .. 16: (I - mu) / sqrt(var + eps_n^2) with mu and
+// var taken over the in-image part of the (2NR+1)^2 box.  FP32 frames: a CTA of
+// 32 x 8 threads stages a 32 x 32 block (four rows per thread) and the NR halo
+// in shared memory (scaled values, zero outside the image, so the boxes are
+// truncated there).  The mean comes from separable sums: row sums over 2NR+1 columns for every staged row, then 2NR+1 of them down
 // each output column.  The variance is the centred sum of (I - mu)^2 over
 // the in-image box (E[I^2] - mu^2 cancels too many digits where the box is
 // flat), with the loop unrolled for NR 1 .. 4 (template NRC) and the box
@@ -82,7 +61,7 @@ template <int NRC, typename TI, typename TS, typename FR>
 __device__ __forceinline__ void ingest_norm_tile(const FR &p)
 {
     pdl_trigger();
-    extern __shared__ float tile[];  // (32 + 2 NR) rows of (32 + 2 NR), then (32 + 2 NR) x 32 row sums
+    extern __shared__ __align__(16) float tile[];  // (32 + 2 NR) rows of (32 + 2 NR), then (32 + 2 NR) x 32 row sums
     const IngestArgs &a = p.get(blockIdx.z);
     const int nr = NRC > 0 ? NRC : a.nr, K = 2 * nr + 1;
     const int TW = 32 + 2 * nr, TH = 32 + 2 * nr;
@@ -170,7 +149,7 @@ __device__ __forceinline__ void ingest_norm_tile(const FR &p)
 template <int NRC, typename ACC, typename TI, typename TS, typename FR>
 __device__ __forceinline__ void ingest_norm_int(const FR &p)
 {
-    extern __shared__ float tile[];
+    extern __shared__ __align__(16) float tile[];
     const IngestArgs &a = p.get(blockIdx.z);
     const int nr = NRC > 0 ? NRC : a.nr, K = 2 * nr + 1;
     const int TW = 32 + 2 * nr, TH = 32 + 2 * nr;
@@ -391,7 +370,7 @@ static cudaError_t ingest_t(const FR &p, const IngestArgs *f, int nframes, cudaS
     }
     dim3 blk(32, 8);
     dim3 grd((W + 31) / 32, (H + 7) / 8, nframes);
-    if (a.nr > 0 && a.nr <= 16) {
+    if (a.nr > 0) {
         const size_t smem = sizeof(float) * (size_t)(32 + 2 * a.nr) * (32 + 2 * a.nr + 32);
         const dim3 grdn((W + 31) / 32, (H + 31) / 32, nframes);
         switch (a.in_type) {

@@ -9,8 +9,8 @@
 //      border replicated in shared memory;
 //   1. a thread walks NROW consecutive rows of one column and forms the five
 //      products of each pixel;
-//   2. vertical window sums of two columns per thread (packed FP32), over the
-//      products;
+//   2. vertical window sums of a column per thread (of two in packed FP32 where
+//      the threads are too few), over the products;
 //   3. horizontal window sums of eight adjacent outputs per thread for all
 //      five channels, the guarded solve and the store, without another pass
 //      through shared memory.

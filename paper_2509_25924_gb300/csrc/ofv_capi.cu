@@ -510,9 +510,10 @@ ofv_status handle_pyramids(ofv_handle *h, const void *const *frames, const int *
 }
 
 // 2-D tensor map of a level image (W x H elements of the storage type, row
-// stride pitch elements) with the block kernel's TMA box for radius kr; no
-// swizzle, out-of-bounds fill unused (only boxes inside the image are
-// copied).  False when the encoder is unavailable or refuses.
+// stride pitch elements) with the iteration kernel's TMA box for radius kr; no
+// swizzle.  Elements of a box outside the image arrive as zero, and the box
+// window's kernels replace those that samples reach by the border's.  False
+// when the encoder is unavailable or refuses.
 bool encode_block_map(CUtensorMap *m, const void *base, int W, int H, int pitch, int store, int kr, int shape, bool var)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder_impl();

@@ -167,7 +167,7 @@ struct IngestArgs {
     float eps_n;
     int prefilter;
 };
-// Ingest nframes (1 or 2) frames in one launch.
+// Ingest nframes (1 .. kMaxFramesPerLaunch) frames in one launch.
 // Kernels after the first start ahead (launch_after) with overlap.
 cudaError_t launch_ingest_frames(const IngestArgs *f, int nframes, int store, cudaStream_t s, bool overlap = false);
 
@@ -175,7 +175,7 @@ struct ReduceArgs {
     const void *src; int Hs, Ws, spitch;
     void *dst; int Hd, Wd, dpitch;
 };
-// Reduce one level of nframes (1 or 2) frames in one launch.
+// Reduce one level of nframes (1 .. kMaxFramesPerLaunch) frames in one launch.
 cudaError_t launch_reduce_frames(const ReduceArgs *f, int nframes, int store, cudaStream_t s, bool overlap = false);
 
 // Any number of frames of any sizes in one launch: f on the host, dev_f the

@@ -108,7 +108,7 @@ struct ofv_handle {
     uint8_t *mask_lvl[ofv::kMaxLevels];
     void *mask_arena;
     int mask_on;
-    // batched entry point: word a persistent launch sets when a dependency
+    // batched entry point: word a batched launch sets when a dependency
     // wait expires (page-locked, mapped), and the layouts whose schedule and
     // tensor maps are in the batch arena
     int *qerr_h, *qerr_d;
