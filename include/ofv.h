@@ -367,8 +367,8 @@ ofv_status ofv_compute_batched(ofv_handle *h, int n, const ofv_pair *pairs, ofv_
  * stage-major over all pairs, else group size), resident CTAs per SM, the
  * output tile edge of the block kernel in px (with ofv_params.tile_edge = 0
  * the autotuner tries the radius's default and alternative edges, except
- * with the Gaussian window or the increment form, which have the default
- * only; a nonzero tile_edge fixes the edge),
+ * with the Gaussian window or the increment form and at KR 1 and 2, which
+ * have the default only; a nonzero tile_edge fixes the edge),
  * duration of its launch in ms, and whether that call tuned.  A
  * handle created with tile_edge set to the reported edge computes, through
  * ofv_compute, bitwise the fields the batch computed. */
