@@ -52,11 +52,12 @@ __global__ void __launch_bounds__(256) k_ingest(const __grid_constant__ FR p)
 // var taken over the in-image part of the (2NR+1)^2 box.  FP32 frames: a CTA of
 // 32 x 8 threads stages a 32 x 32 block (four rows per thread) and the NR halo
 // in shared memory (scaled values, zero outside the image, so the boxes are
-// truncated there).  The mean comes from separable sums: row sums over 2NR+1 columns for every staged row, then 2NR+1 of them down
-// each output column.  The variance is the centred sum of (I - mu)^2 over
-// the in-image box (E[I^2] - mu^2 cancels too many digits where the box is
-// flat), with the loop unrolled for NR 1 .. 4 (template NRC) and the box
-// bounds tested only for pixels within NR of the border.
+// truncated there).  The mean comes from separable sums: row sums over 2NR+1
+// columns for every staged row, then 2NR+1 of them down each output column.
+// The variance is the centred sum of (I - mu)^2 over the in-image box
+// (E[I^2] - mu^2 cancels too many digits where the box is flat), with the loop
+// unrolled for NR 1 .. 4 (template NRC) and the box bounds tested only for
+// pixels within NR of the border.
 template <int NRC, typename TI, typename TS, typename FR>
 __device__ __forceinline__ void ingest_norm_tile(const FR &p)
 {
